@@ -290,7 +290,7 @@ emrt_status emrt_channel_multi(emrt_scene sc, const emrt_paths *paths, const emr
  * given dloss_dh [n_tx][n_rx][2] (d loss / d Re h, d loss / d Im h),
  * accumulates (overwrites) grad_eps [n_mat], grad_sigma [n_mat] and
  * grad_tx [n_tx][3].  Reflection points are recomputed, not stored.  A
- * non-finite amplitude or tangent (e.g. NaN material parameters) makes the
+ * non-finite amplitude or derivative (e.g. NaN material parameters) makes the
  * next emrt_sync return EMRT_ERR_DEVICE. */
 emrt_status emrt_channel_backward(emrt_scene sc, const emrt_paths *paths,
                                   const emrt_materials *m, double freq_hz,
@@ -306,7 +306,7 @@ emrt_status emrt_channel_backward(emrt_scene sc, const emrt_paths *paths,
  * it is a library service.
  *
  * Same arguments and results as emrt_channel_backward, but the per-path
- * tangent scratch lives in a fixed device array compiled into libemrt.so
+ * derivative scratch lives in a fixed device array compiled into libemrt.so
  * (EMRT_NOALLOC_MAX_PATHS x 11 doubles, 5.8 MB, held by every GPU that loads
  * the library until the process exits) instead of scene-owned memory, and the
  * call allocates nothing: no cudaMalloc, cudaFree or allocating library
@@ -323,7 +323,7 @@ emrt_status emrt_channel_backward(emrt_scene sc, const emrt_paths *paths,
  *    gradients; order them on one stream.  The array keeps the last call's
  *    contents; each call overwrites every entry it reads, so no clearing is
  *    needed;
- *  - a non-finite amplitude or tangent makes the next emrt_sync return
+ *  - a non-finite amplitude or derivative makes the next emrt_sync return
  *    EMRT_ERR_DEVICE, as for emrt_channel_backward. */
 #define EMRT_NOALLOC_MAX_PATHS 65536u
 emrt_status emrt_channel_backward_noalloc(emrt_scene sc, const emrt_paths *paths,

@@ -880,7 +880,7 @@ emrt_status emrt_channel_backward(emrt_scene s, const emrt_paths *paths, const e
 }  // extern "C"
 
 // ---------------------------------------------------------------------------
-// Allocation-free adjoint: the per-path tangent scratch is this file-scope
+// Allocation-free adjoint: the per-path derivative scratch is this file-scope
 // device array (EMRT_NOALLOC_MAX_PATHS x 11 doubles).  Host code must not use
 // the symbol `g_noalloc_contrib` as an address: it is a host-side stand-in.
 // Its device address is looked up once per device, with that device current,

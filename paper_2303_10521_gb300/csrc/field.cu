@@ -2,12 +2,10 @@
 // Sec. V-D) and the adjoint of the coherent sums with respect to material
 // permittivity, conductivity and transmitter position.
 //
-// One generic routine computes the field of a path for a scalar type T.  With
-// T = double it is the forward kernel; with T = Dual<N> (value plus N
-// tangents) the same arithmetic carries derivatives with respect to the
-// transmitter coordinates and the (eps_r, sigma) of every bounce, so the
-// adjoint recomputes reflection points instead of storing Jacobians.  Path
-// length and phase are accumulated in FP64 (L / lambda formed in double).
+// The forward routines compute the field of a path in FP64; the adjoint
+// recomputes a path's points, basis vectors and coefficients instead of
+// storing them and runs the same steps backwards.  Path length and phase are
+// accumulated in FP64 (L / lambda formed in double).
 #include "field.cuh"
 
 namespace emrt {
@@ -19,87 +17,12 @@ constexpr double kEps0 = 8.8541878128e-12;
 constexpr double kPi = 3.14159265358979323846;
 
 // ---------------------------------------------------------------------------
-// scalar abstraction
-template <int N>
-struct Dual {
-  double v;
-  double d[N];
-  __device__ Dual() {}
-  __device__ Dual(double x) : v(x) {
-#pragma unroll
-    for (int i = 0; i < N; i++) d[i] = 0.0;
-  }
-};
-
+// scalar functions of the generic field routines
 __device__ inline double val(double x) { return x; }
-template <int N> __device__ inline double val(const Dual<N> &x) { return x.v; }
-
-template <int N> __device__ inline Dual<N> operator+(const Dual<N> &a, const Dual<N> &b) {
-  Dual<N> r; r.v = a.v + b.v;
-#pragma unroll
-  for (int i = 0; i < N; i++) r.d[i] = a.d[i] + b.d[i];
-  return r;
-}
-template <int N> __device__ inline Dual<N> operator-(const Dual<N> &a, const Dual<N> &b) {
-  Dual<N> r; r.v = a.v - b.v;
-#pragma unroll
-  for (int i = 0; i < N; i++) r.d[i] = a.d[i] - b.d[i];
-  return r;
-}
-template <int N> __device__ inline Dual<N> operator-(const Dual<N> &a) {
-  Dual<N> r; r.v = -a.v;
-#pragma unroll
-  for (int i = 0; i < N; i++) r.d[i] = -a.d[i];
-  return r;
-}
-template <int N> __device__ inline Dual<N> operator*(const Dual<N> &a, const Dual<N> &b) {
-  Dual<N> r; r.v = a.v * b.v;
-#pragma unroll
-  for (int i = 0; i < N; i++) r.d[i] = a.d[i] * b.v + a.v * b.d[i];
-  return r;
-}
-template <int N> __device__ inline Dual<N> operator/(const Dual<N> &a, const Dual<N> &b) {
-  Dual<N> r; r.v = a.v / b.v;
-  double ib = 1.0 / b.v;
-#pragma unroll
-  for (int i = 0; i < N; i++) r.d[i] = (a.d[i] - r.v * b.d[i]) * ib;
-  return r;
-}
-template <int N> __device__ inline Dual<N> operator+(const Dual<N> &a, double b) { return a + Dual<N>(b); }
-template <int N> __device__ inline Dual<N> operator-(const Dual<N> &a, double b) { return a - Dual<N>(b); }
-template <int N> __device__ inline Dual<N> operator-(double a, const Dual<N> &b) { return Dual<N>(a) - b; }
-template <int N> __device__ inline Dual<N> operator*(const Dual<N> &a, double b) {
-  Dual<N> r; r.v = a.v * b;
-#pragma unroll
-  for (int i = 0; i < N; i++) r.d[i] = a.d[i] * b;
-  return r;
-}
-template <int N> __device__ inline Dual<N> operator*(double b, const Dual<N> &a) { return a * b; }
-template <int N> __device__ inline Dual<N> operator/(const Dual<N> &a, double b) { return a * (1.0 / b); }
-template <int N> __device__ inline Dual<N> operator/(double a, const Dual<N> &b) { return Dual<N>(a) / b; }
-
 __device__ inline double tsqrt(double x) { return sqrt(x); }
-template <int N> __device__ inline Dual<N> tsqrt(const Dual<N> &a) {
-  Dual<N> r; r.v = sqrt(a.v);
-  double h = r.v > 0.0 ? 0.5 / r.v : 0.0;
-#pragma unroll
-  for (int i = 0; i < N; i++) r.d[i] = a.d[i] * h;
-  return r;
-}
 __device__ inline double tabs(double x) { return fabs(x); }
-template <int N> __device__ inline Dual<N> tabs(const Dual<N> &a) { return a.v < 0.0 ? -a : a; }
 __device__ inline double tfrac(double x) { return x - floor(x); }
-template <int N> __device__ inline Dual<N> tfrac(const Dual<N> &a) {
-  Dual<N> r = a; r.v = a.v - floor(a.v); return r;
-}
 __device__ inline void tsincos(double x, double &s, double &c) { sincos(x, &s, &c); }
-template <int N> __device__ inline void tsincos(const Dual<N> &x, Dual<N> &s, Dual<N> &c) {
-  double sv, cv;
-  sincos(x.v, &sv, &cv);
-  s.v = sv; c.v = cv;
-#pragma unroll
-  for (int i = 0; i < N; i++) { s.d[i] = x.d[i] * cv; c.d[i] = -x.d[i] * sv; }
-}
 
 template <typename T> struct V3 { T x, y, z; };
 template <typename T> __device__ inline V3<T> mk3(T x, T y, T z) { V3<T> r; r.x = x; r.y = y; r.z = z; return r; }
@@ -201,7 +124,7 @@ __device__ inline void load_geom(const GeomView &g, const uint32_t *rec, PathGeo
 
 // Geometry of one path (frequency-independent): image points, reflection
 // points, the unfolded length L and the unit direction kh[q] of every leg.
-// tx: transmitter position (seeded with tangents by the caller).
+// tx: transmitter position.
 template <typename T>
 __device__ inline void path_geometry(const PathGeom &P, V3<T> tx, V3<double> rx, T &Lout,
                                      V3<T> *kh) {
@@ -280,15 +203,6 @@ __device__ inline void path_transport(const PathGeom &P, const V3<T> *kh, T L, c
   tsincos(ph, sp, cp);
   T sc = T(lam / (4.0 * kPi)) / L;
   amp = cscale(rcv * cx<T>(cp, sp), sc);
-}
-
-// Field of one path at one frequency (geometry and transport).
-template <typename T>
-__device__ inline void path_field(const PathGeom &P, V3<T> tx, V3<double> rx, const T *epsr,
-                                  const T *sig, const double *gam, bool const_gamma, double freq,
-                                  Cx<T> &amp, T &Lout, V3<T> *kh) {
-  path_geometry<T>(P, tx, rx, Lout, kh);
-  path_transport<T>(P, kh, Lout, epsr, sig, gam, const_gamma, freq, amp);
 }
 
 // frequency q of a set (kernel parameters; no dynamic indexing)
@@ -437,63 +351,323 @@ __global__ void k_rx_power(uint32_t n_tx, uint32_t n_rx, double pt, FreqSet fs) 
 }
 
 // ---------------------------------------------------------------------------
-// adjoint: per path, tangents for tx (3) and (eps_r, sigma) of each bounce
+// adjoint: per path, the derivative of the loss with respect to tx (3) and
+// (eps_r, sigma) of each bounce, in reverse mode.
+//
+// Bound by the latency of FP64 instructions: on GB300 a warp issues one every
+// 64 cycles (19 with four warps an SM), whatever the active lanes and the
+// independent chains, so a path's time is the number of FP64 instructions its
+// warp executes.  Four lanes share a path, lane q its bounce q (and leg q):
+// what belongs to one bounce -- incidence basis, Fresnel coefficients and
+// their derivatives, a leg's length and direction -- runs for all bounces at
+// once, only the short chains along the path (images, reflection points, the
+// transported field and its cotangent) run in order, in all four lanes alike.
+// The lanes exchange through shared memory.  District, about 3k paths: 960 us
+// with 11 forward-mode tangents per path in one thread -> 52 us.
 constexpr int kTan = 3 + 2 * EMRT_MAX_DEPTH;
-constexpr int kAdjBlock = 64;
+constexpr int kAdjBlock = 32, kAdjPaths = kAdjBlock / EMRT_MAX_DEPTH;
+static_assert(EMRT_MAX_DEPTH == 4, "one lane per bounce: a path is four lanes");
 
-__global__ void __launch_bounds__(kAdjBlock) k_field_tangents(GeomView g, MatView m,
-                                                              const uint32_t *rec, const uint32_t *n,
-                                                              uint32_t cap, double freq,
-                                                              const double *dloss_dh, uint32_t n_rx,
-                                                              double *contrib, Counters *ctr) {
-  using D = Dual<kTan>;
-  uint32_t cnt = min(*n, cap);
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
-    PathGeom P;
-    const uint32_t *r = rec + 8ull * i;
-    uint32_t tx = r[0], rx = r[1];
+using V = V3<double>;
+using C = Cx<double>;
+struct AdjPath {                      // one path's exchange between its lanes
+  V n[EMRT_MAX_DEPTH];                // face normals
+  double d[EMRT_MAX_DEPTH];           // face offsets
+  V kh[EMRT_MAX_DEPTH + 1];           // unit leg directions
+  double len[EMRT_MAX_DEPTH + 1];     // leg lengths
+  V sv[EMRT_MAX_DEPTH], pin[EMRT_MAX_DEPTH], pout[EMRT_MAX_DEPTH];
+  C gs[EMRT_MAX_DEPTH], gp[EMRT_MAX_DEPTH];
+  V kin_bar[EMRT_MAX_DEPTH], kout_bar[EMRT_MAX_DEPTH];
+  V leg_bar[EMRT_MAX_DEPTH + 1];      // cotangent of every leg vector
+};
+
+__device__ inline V operator*(const V &a, double s) { return mk3<double>(a.x * s, a.y * s, a.z * s); }
+__device__ inline C conjc(const C &a) { return cx<double>(a.re, -a.im); }
+// real part of a conj(b): the cotangent of a real factor whose product has
+// cotangent a, the other factor being b
+__device__ inline double rdot(const C &a, const C &b) { return a.re * b.re + a.im * b.im; }
+// cotangent of polar(k) (u = polar(k)) pulled back to k
+__device__ inline V polar_bar(const V &k, const V &u, const V &ub) {
+  const V p = mk3<double>(-k.z * k.x, -k.z * k.y, 1.0 - k.z * k.z);
+  const double n = sqrt(dot(p, p));
+  if (n < 1e-12) return mk3<double>(0.0, 0.0, 0.0);  // constant axis
+  const V pb = (ub - u * dot(u, ub)) * (1.0 / n);
+  return mk3<double>(-k.z * pb.x, -k.z * pb.y, -k.x * pb.x - k.y * pb.y - 2.0 * k.z * pb.z);
+}
+
+__global__ void __launch_bounds__(kAdjBlock) k_field_adjoint(GeomView g, MatView m,
+                                                             const uint32_t *rec, const uint32_t *n,
+                                                             uint32_t cap, double freq,
+                                                             const double *dloss_dh, uint32_t n_rx,
+                                                             double *contrib, Counters *ctr) {
+  __shared__ AdjPath s_path[kAdjPaths];
+  constexpr int K = EMRT_MAX_DEPTH;
+  const uint32_t cnt = min(*n, cap);
+  const int q = threadIdx.x % K;
+  AdjPath &S = s_path[threadIdx.x / K];
+  const double lam = kC / freq, kappa = 1.0 / (2.0 * kPi * freq * kEps0);
+  for (uint32_t base = blockIdx.x * kAdjPaths; base < cnt; base += gridDim.x * kAdjPaths) {
+    const uint32_t i = base + threadIdx.x / K;
+    const uint32_t *r = rec + 8ull * min(i, cnt - 1u);
+    const bool live = i < cnt, ok = live && record_ok(g, r);
+    const uint32_t tx = r[0], rx = r[1];
+    const int k = ok ? (int)(r[2] & 15u) : 0;
     double *c = contrib + (size_t)kTan * i;
-    if (!record_ok(g, r)) {
-      for (int t = 0; t < kTan; t++) c[t] = 0.0;
-      continue;
+    double eps = 1.0, sig = 0.0, gam = 0.0;
+    if (q < k) {
+      PathGeom P;
+      load_geom(g, r, P);
+      V nq = mk3<double>(0.0, 0.0, 0.0);
+      double dq = 0.0;
+      uint32_t mat = 0;
+#pragma unroll
+      for (int j = 0; j < K; j++)
+        if (j == q) {
+          nq = mk3<double>(P.n[j][0], P.n[j][1], P.n[j][2]);
+          dq = P.d[j];
+          mat = P.mat[j];
+        }
+      S.n[q] = nq;
+      S.d[q] = dq;
+      mat = min(mat, m.n_mat - 1);
+      eps = m.eps_r[mat];
+      sig = m.sigma[mat];
+      gam = m.gamma ? m.gamma[mat] : 0.0;
     }
-    load_geom(g, r, P);
-    D epsr[EMRT_MAX_DEPTH], sig[EMRT_MAX_DEPTH];
-    double gam[EMRT_MAX_DEPTH];
-    for (uint32_t q = 0; q < P.k; q++) {
-      uint32_t mm = min(P.mat[q], m.n_mat - 1);
-      epsr[q] = D(m.eps_r[mm]);
-      epsr[q].d[3 + 2 * q] = 1.0;
-      sig[q] = D(m.sigma[mm]);
-      sig[q].d[4 + 2 * q] = 1.0;
-      gam[q] = m.gamma ? m.gamma[mm] : 0.0;
+    __syncwarp();
+    // images of the transmitter, reflection points from the receiver back
+    V I[K + 1], Q[K + 2], Dv[K + 1];
+    double tq[K + 1], den[K + 1];
+    {
+      const float3 t3 = ok ? f3(g.tx_pos[tx]) : make_float3(0.f, 0.f, 0.f);
+      const float3 r3 = ok ? f3(g.rx_pos[rx]) : make_float3(1.f, 0.f, 0.f);
+      I[0] = mk3<double>(t3.x, t3.y, t3.z);
+#pragma unroll
+      for (int j = 0; j < K; j++)
+        if (j < k) I[j + 1] = I[j] - S.n[j] * (2.0 * (dot(S.n[j], I[j]) - S.d[j]));
+      V next = mk3<double>(r3.x, r3.y, r3.z);
+#pragma unroll
+      for (int j = K; j >= 0; j--) {  // Q[j + 1] of the legs j = k .. 0
+        if (j > k) continue;
+        Q[j + 1] = next;
+        if (j == 0) {
+          Q[0] = I[0];
+        } else {
+          Dv[j] = next - I[j];
+          den[j] = dot(S.n[j - 1], Dv[j]);
+          tq[j] = (S.d[j - 1] - dot(S.n[j - 1], I[j])) / den[j];
+          next = I[j] + Dv[j] * tq[j];
+        }
+      }
     }
-    float3 t3 = f3(g.tx_pos[tx]), r3 = f3(g.rx_pos[rx]);
-    V3<D> txp = mk3<D>(D(t3.x), D(t3.y), D(t3.z));
-    txp.x.d[0] = 1.0; txp.y.d[1] = 1.0; txp.z.d[2] = 1.0;
-    V3<double> rxp = mk3<double>(r3.x, r3.y, r3.z);
-    Cx<D> a;
-    D L;
-    V3<D> kh[EMRT_MAX_DEPTH + 1];
-    path_field<D>(P, txp, rxp, epsr, sig, gam, m.const_gamma != 0, freq, a, L, kh);
-    const double *gh = dloss_dh + 2ull * (tx * n_rx + rx);
-    double gx = gh[0], gy = gh[1];
-    bool finite = isfinite(a.re.v) && isfinite(a.im.v);
-    for (int t = 0; t < kTan; t++) {
-      c[t] = gx * a.re.d[t] + gy * a.im.d[t];
-      finite = finite && isfinite(c[t]);
+    // legs: lane q takes leg q (and lane 0 leg 4)
+#pragma unroll
+    for (int j = 0; j <= K; j++)
+      if (j <= k && j % K == q) {
+        const V D = Q[j + 1] - Q[j];
+        const double l = sqrt(dot(D, D));
+        S.len[j] = l;
+        S.kh[j] = D * (1.0 / l);
+      }
+    __syncwarp();
+    double L = 0.0;
+#pragma unroll
+    for (int j = 0; j <= K; j++)
+      if (j <= k) L = L + S.len[j];
+    // the lane's bounce: incidence basis and Fresnel coefficients
+    V kin, kout, nq, sv, axis;
+    C ec, root;
+    double cn = 0.0, cos_t = 0.0, c_inv = 1.0;
+    if (q < k) {
+      nq = S.n[q];
+      kin = S.kh[q];
+      kout = S.kh[q + 1];
+      cn = dot(kin, nq);
+      cos_t = fabs(cn);
+      axis = nq;
+      sv = cross(kin, axis);
+      double s2 = dot(sv, sv);
+      if (s2 < 1e-24) {  // normal incidence: any s orthogonal to kin
+        axis = mk3<double>(1.0, 0.0, 0.0);
+        sv = cross(kin, axis);
+        s2 = dot(sv, sv);
+        if (s2 < 1e-12) {
+          axis = mk3<double>(0.0, 1.0, 0.0);
+          sv = cross(kin, axis);
+          s2 = dot(sv, sv);
+        }
+      }
+      c_inv = 1.0 / sqrt(s2);
+      sv = sv * c_inv;
+      S.sv[q] = sv;
+      S.pin[q] = cross(sv, kin);
+      S.pout[q] = cross(sv, kout);
+      if (m.const_gamma) {
+        S.gs[q] = cx<double>(-gam, 0.0);
+        S.gp[q] = cx<double>(gam, 0.0);
+      } else {
+        ec = cx<double>(eps, -sig * kappa);
+        root = csqrt_p(cx<double>(ec.re - (1.0 - cos_t * cos_t), ec.im));
+        const C ct = cx<double>(cos_t, 0.0), u = cscale(ec, cos_t);
+        S.gs[q] = (ct - root) / (ct + root);
+        S.gp[q] = (u - root) / (u + root);
+      }
     }
-    // a non-finite amplitude or tangent (e.g. NaN material parameters) is
-    // reported as for the forward field
-    if (!finite) atomicOr(&ctr->err, ERR_NONFINITE);
+    __syncwarp();
+    // transported field; lane q keeps its bounce's incoming field and parts
+    const V p0 = polar(S.kh[0]);
+    CV3<double> E, Ein;
+    E.x = cx<double>(p0.x, 0.0);
+    E.y = cx<double>(p0.y, 0.0);
+    E.z = cx<double>(p0.z, 0.0);
+    Ein = E;
+    C es = cx<double>(0.0, 0.0), ep = es, ga = es, gb = es;
+#pragma unroll
+    for (int j = 0; j < K; j++)
+      if (j < k) {
+        const V s = S.sv[j], po = S.pout[j];
+        const C e0 = cdot(E, s), e1 = cdot(E, S.pin[j]);
+        const C a = S.gs[j] * e0, b = S.gp[j] * e1;
+        if (j == q) {
+          Ein = E;
+          es = e0;
+          ep = e1;
+          ga = a;
+          gb = b;
+        }
+        E.x = cscale(a, s.x) + cscale(b, po.x);
+        E.y = cscale(a, s.y) + cscale(b, po.y);
+        E.z = cscale(a, s.z) + cscale(b, po.z);
+      }
+    const V kl = S.kh[k], pr = polar(kl);
+    const C rcv = cdot(E, pr);
+    const double ph = tfrac(L * (1.0 / lam)) * (-2.0 * kPi);
+    double sp, cp;
+    sincos(ph, &sp, &cp);
+    const double sc = (lam / (4.0 * kPi)) / L;
+    const C w = cx<double>(cp, sp), v = rcv * w, amp = cscale(v, sc);
+    // cotangents: of the amplitude, of the phase and spreading (to L), of
+    // the received field
+    const double *gh = dloss_dh + 2ull * (ok ? (size_t)tx * n_rx + rx : 0);
+    const C ab = cx<double>(gh[0], gh[1]);
+    const C vb = cscale(ab, sc), rb = vb * conjc(w);
+    const double Lb = (vb.im * v.re - vb.re * v.im) * (-2.0 * kPi / lam) - rdot(ab, amp) / L;
+    CV3<double> Eb;
+    Eb.x = cscale(rb, pr.x);
+    Eb.y = cscale(rb, pr.y);
+    Eb.z = cscale(rb, pr.z);
+    const V prb = mk3<double>(rdot(rb, E.x), rdot(rb, E.y), rdot(rb, E.z));
+    CV3<double> Eout = Eb;  // cotangent of the field leaving the lane's bounce
+#pragma unroll
+    for (int j = K - 1; j >= 0; j--)
+      if (j < k) {
+        const V s = S.sv[j], pi = S.pin[j];
+        if (j == q) Eout = Eb;
+        const C esb = cdot(Eb, s) * conjc(S.gs[j]), epb = cdot(Eb, S.pout[j]) * conjc(S.gp[j]);
+        Eb.x = cscale(esb, s.x) + cscale(epb, pi.x);
+        Eb.y = cscale(esb, s.y) + cscale(epb, pi.y);
+        Eb.z = cscale(esb, s.z) + cscale(epb, pi.z);
+      }
+    // the lane's bounce, backwards
+    double eps_b = 0.0, sig_b = 0.0;
+    if (q < k) {
+      const V pin = S.pin[q], pout = S.pout[q];
+      const C abar = cdot(Eout, sv), bbar = cdot(Eout, pout);
+      const C esb = abar * conjc(S.gs[q]), epb = bbar * conjc(S.gp[q]);
+      V svb = mk3<double>(rdot(Eout.x, ga) + rdot(esb, Ein.x), rdot(Eout.y, ga) + rdot(esb, Ein.y),
+                          rdot(Eout.z, ga) + rdot(esb, Ein.z));
+      const V poutb = mk3<double>(rdot(Eout.x, gb), rdot(Eout.y, gb), rdot(Eout.z, gb));
+      const V pinb = mk3<double>(rdot(epb, Ein.x), rdot(epb, Ein.y), rdot(epb, Ein.z));
+      // pin = sv x kin, pout = sv x kout
+      svb = svb + cross(kin, pinb) + cross(kout, poutb);
+      V kinb = cross(pinb, sv);
+      S.kout_bar[q] = cross(poutb, sv);
+      // sv = unit(kin x axis)
+      const V cb = (svb - sv * dot(sv, svb)) * c_inv;
+      kinb = kinb + cross(axis, cb);
+      if (!m.const_gamma) {
+        const C gsb = abar * conjc(es), gpb = bbar * conjc(ep);
+        const C ct = cx<double>(cos_t, 0.0), u = cscale(ec, cos_t);
+        const C ds = ct + root, dp = u + root;
+        // d gs = (2 root d ct - 2 ct d root) / ds^2, gp alike with u for ct
+        const C hs = gsb * conjc(cx<double>(2.0, 0.0) / (ds * ds));
+        const C hp = gpb * conjc(cx<double>(2.0, 0.0) / (dp * dp));
+        const C ub = hp * conjc(root);
+        const C rootb = cx<double>(0.0, 0.0) - (cscale(hs, cos_t) + hp * conjc(u));
+        C zb = cx<double>(0.0, 0.0);
+        if (root.re != 0.0 || root.im != 0.0) zb = rootb * conjc(cx<double>(0.5, 0.0) / root);
+        const C ecb = cscale(ub, cos_t) + zb;
+        const double ctb = rdot(hs, root) + rdot(ub, ec) + 2.0 * cos_t * zb.re;
+        eps_b = ecb.re;
+        sig_b = -kappa * ecb.im;
+        kinb = kinb + nq * (cn < 0.0 ? -ctb : ctb);
+      }
+      S.kin_bar[q] = kinb;
+    }
+    __syncwarp();
+    // legs, backwards: unit directions and lengths to leg vectors
+#pragma unroll
+    for (int j = 0; j <= K; j++)
+      if (j <= k && j % K == q) {
+        const V kj = S.kh[j];
+        V kb = mk3<double>(0.0, 0.0, 0.0);
+        if (j < k) kb = kb + S.kin_bar[j];
+        if (j > 0) kb = kb + S.kout_bar[j - 1];
+        if (j == 0) kb = kb + polar_bar(kj, p0, mk3<double>(Eb.x.re, Eb.y.re, Eb.z.re));
+        if (j == k) kb = kb + polar_bar(kj, pr, prb);
+        S.leg_bar[j] = (kb - kj * dot(kj, kb)) * (1.0 / S.len[j]) + kj * Lb;
+      }
+    __syncwarp();
+    // reflection points and images, backwards, to the transmitter
+    V Ib[K + 1], Qb = mk3<double>(0.0, 0.0, 0.0);
+#pragma unroll
+    for (int j = 1; j <= K; j++) {
+      if (j > k) continue;
+      Qb = Qb + S.leg_bar[j - 1] - S.leg_bar[j];
+      const V nj = S.n[j - 1];
+      const double tb = dot(Qb, Dv[j]) / den[j];
+      const V Db = Qb * tq[j] - nj * (tb * tq[j]);
+      Ib[j] = Qb - nj * tb - Db;
+      Qb = Db;
+    }
+    V txb = mk3<double>(0.0, 0.0, 0.0) - S.leg_bar[0];
+    V acc = mk3<double>(0.0, 0.0, 0.0);
+#pragma unroll
+    for (int j = K; j >= 1; j--) {
+      if (j > k) continue;
+      acc = acc + Ib[j];
+      acc = acc - S.n[j - 1] * (2.0 * dot(S.n[j - 1], acc));
+    }
+    txb = txb + acc;
+    if (live) {
+      const bool tx_fin = isfinite(txb.x) && isfinite(txb.y) && isfinite(txb.z);
+      if (!ok) txb = mk3<double>(0.0, 0.0, 0.0);
+      if (q == 0) {
+        c[0] = txb.x;
+        c[1] = txb.y;
+        c[2] = txb.z;
+      }
+      c[3 + 2 * q] = eps_b;
+      c[4 + 2 * q] = sig_b;
+      // a non-finite amplitude or derivative (e.g. NaN material parameters)
+      // is reported as for the forward field
+      if (ok && !(isfinite(amp.re) && isfinite(amp.im) && tx_fin && isfinite(eps_b) &&
+                  isfinite(sig_b)))
+        atomicOr(&ctr->err, ERR_NONFINITE);
+    }
+    __syncwarp();
   }
 }
 
-// one block per gradient entry, fixed-order sum over paths
-__global__ void k_grad_reduce(GeomView g, MatView m, const uint32_t *rec, const uint32_t *n,
+// One block per gradient entry, fixed-order sum over paths.  Bound by the
+// latency of a thread's dependent loads (record, face material,
+// contribution) per path it visits: 1024 threads visit a quarter of the paths
+// each that 256 would.
+constexpr int kGradBlock = 1024;
+__global__ void __launch_bounds__(kGradBlock) k_grad_reduce(GeomView g, MatView m, const uint32_t *rec, const uint32_t *n,
                               uint32_t cap, const double *contrib, double *grad_eps,
                               double *grad_sigma, double *grad_tx) {
-  __shared__ double sh[256];
+  __shared__ double sh[kGradBlock];
   uint32_t cnt = min(*n, cap);
   uint32_t pid = blockIdx.x;  // [0, n_mat) eps, [n_mat, 2 n_mat) sigma, then tx*3+c
   double s = 0.0;
@@ -516,7 +690,7 @@ __global__ void k_grad_reduce(GeomView g, MatView m, const uint32_t *rec, const 
   }
   sh[threadIdx.x] = s;
   __syncthreads();
-  for (int o = 128; o; o >>= 1) {
+  for (int o = kGradBlock / 2; o; o >>= 1) {
     if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
     __syncthreads();
   }
@@ -760,16 +934,17 @@ void launch_channel(const GeomView &g, MatView m, const uint32_t *rec, const uin
     emrt::note_launch(), k_rx_power<<<dim3(ceil_div(n_rx, 256), fs.n), 256, 0, s>>>(n_tx, n_rx, tx_power_w, fs);
 }
 
-int adjoint_grid() { return 152 * 4; }
+// blocks of one warp (eight paths): sixteen an SM
+int adjoint_grid() { return 152 * 16; }
 
 void launch_field_adjoint(const GeomView &g, MatView m, const uint32_t *rec, const uint32_t *n,
                           uint32_t cap, double freq, const double *dloss_dh, uint32_t n_rx,
                           double *contrib, double *grad_eps, double *grad_sigma, double *grad_tx,
                           Counters *ctr, cudaStream_t s) {
-  emrt::note_launch(), k_field_tangents<<<adjoint_grid(), kAdjBlock, 0, s>>>(g, m, rec, n, cap, freq, dloss_dh, n_rx,
-                                                        contrib, ctr);
+  emrt::note_launch(), k_field_adjoint<<<adjoint_grid(), kAdjBlock, 0, s>>>(g, m, rec, n, cap, freq, dloss_dh, n_rx,
+                                                       contrib, ctr);
   uint32_t n_par = 2 * m.n_mat + 3 * g.n_tx;
-  emrt::note_launch(), k_grad_reduce<<<n_par, 256, 0, s>>>(g, m, rec, n, cap, contrib, grad_eps, grad_sigma, grad_tx);
+  emrt::note_launch(), k_grad_reduce<<<n_par, kGradBlock, 0, s>>>(g, m, rec, n, cap, contrib, grad_eps, grad_sigma, grad_tx);
 }
 
 }  // namespace emrt
