@@ -10,6 +10,7 @@
 
 #include "bvh.cuh"
 #include "field.cuh"
+#include "lbvh.cuh"
 #include "trace.cuh"
 #include "scene.cuh"
 
@@ -74,11 +75,12 @@ __global__ void k_half(const float *h, uint32_t V, float4 *out) {
   if (v < V) out[v] = make_float4(h[3 * v], h[3 * v + 1], h[3 * v + 2], 0.f);
 }
 
-// per-frame state: box corners in float32 arithmetic, receivers, transmitters
+// per-frame state: box corners in float32 arithmetic, receivers, transmitters;
+// codes: also the codes of the trees built together (vehicles, receivers)
 __global__ void k_update(const float *vp, const float *vv, const float4 *half, uint32_t V,
                          float4 *lo, float4 *hi, float4 *vel, const float *rp, const float *rv,
                          uint32_t R, float4 *rxp, float4 *rxv, const float *tp, const float *tv,
-                         uint32_t X, float4 *txp, float4 *txv) {
+                         uint32_t X, float4 *txp, float4 *txv, const float4 *bb, FrameTreesBuf trees, bool codes) {
   uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < V) {
     float4 h = half[i];
@@ -86,10 +88,12 @@ __global__ void k_update(const float *vp, const float *vv, const float4 *half, u
     lo[i] = make_float4(__fsub_rn(x, h.x), __fsub_rn(y, h.y), __fsub_rn(z, h.z), 0.f);
     hi[i] = make_float4(__fadd_rn(x, h.x), __fadd_rn(y, h.y), __fadd_rn(z, h.z), 0.f);
     vel[i] = vv ? make_float4(vv[3 * i], vv[3 * i + 1], vv[3 * i + 2], 0.f) : make_float4(0, 0, 0, 0);
+    if (codes) frame_code(trees, i, true, lo[i], hi[i], bb);
   }
   if (i < R) {
     rxp[i] = make_float4(rp[3 * i], rp[3 * i + 1], rp[3 * i + 2], 0.f);
     rxv[i] = rv ? make_float4(rv[3 * i], rv[3 * i + 1], rv[3 * i + 2], 0.f) : make_float4(0, 0, 0, 0);
+    if (codes) frame_code(trees, V + i, false, rxp[i], rxp[i], bb);
   }
   if (i < X) {
     txp[i] = make_float4(tp[3 * i], tp[3 * i + 1], tp[3 * i + 2], 0.f);
@@ -273,8 +277,11 @@ emrt_status emrt_scene_create(const emrt_scene_desc *d, emrt_stream stream, emrt
   // the per-frame builds report a barrier that gave up through the
   // scene's error word (read by the next emrt_sync)
   s->dyn.err_word = s->rxb.err_word = s->txb.err_word = s->mix.err_word = &s->ctr->err;
-  if ((e = grow(&s->mix_lo, c, s->V + s->max_rx))) return fail(e); c = 0;
-  if ((e = grow(&s->mix_hi, c, s->V + s->max_rx))) return fail(e); c = 0;
+  if ((e = frame_trees_alloc(s->frame_trees, s->V + s->max_rx))) return fail(e);
+  if (s->V + s->max_rx > kFrameTreesMax) {
+    if ((e = grow(&s->mix_lo, c, s->V + s->max_rx))) return fail(e); c = 0;
+    if ((e = grow(&s->mix_hi, c, s->V + s->max_rx))) return fail(e); c = 0;
+  }
   uint32_t V1 = std::max(s->V, 1u);
   if ((e = grow(&s->veh_half, c, V1))) return fail(e); c = 0;
   if ((e = grow(&s->veh_lo, c, V1))) return fail(e); c = 0;
@@ -302,6 +309,7 @@ void emrt_scene_destroy(emrt_scene s) {
   cudaFree(s->face_plane); cudaFree(s->face_info); cudaFree(s->face_vert); cudaFree(s->bbox);
   bvh_free(s->stat); bvh_free(s->dyn); bvh_free(s->rxb); bvh_free(s->txb); bvh_free(s->mix);
   cudaFree(s->mix_lo); cudaFree(s->mix_hi);
+  frame_trees_free(s->frame_trees);
   cudaFree(s->src_pos);
   cudaFree(s->veh_half); cudaFree(s->veh_lo); cudaFree(s->veh_hi); cudaFree(s->veh_vel);
   cudaFree(s->rx_pos); cudaFree(s->rx_vel); cudaFree(s->tx_pos); cudaFree(s->tx_vel);
@@ -346,24 +354,36 @@ emrt_status emrt_scene_update_dynamic(emrt_scene s, const float *veh_pos, const 
   s->n_rx = n_rx;
   s->n_tx = n_tx;
   uint32_t m = std::max(s->V, std::max(n_rx, n_tx));
+  const uint32_t nm = s->V + n_rx;
+  const bool together = nm <= kFrameTreesMax;
+  if (together) CK(cudaMemsetAsync(s->frame_trees.count, 0, sizeof(uint32_t) * 2 * kTreeBins, st));
   emrt::note_launch(), k_update<<<ceil_div(m, 256), 256, 0, st>>>(veh_pos, veh_vel, s->veh_half, s->V, s->veh_lo,
                                              s->veh_hi, s->veh_vel, rx_pos, rx_vel, n_rx,
                                              s->rx_pos, s->rx_vel, tx_pos, tx_vel, n_tx, s->tx_pos,
-                                             s->tx_vel);
-  // the three per-frame trees are independent small builds (a few tens of
-  // blocks per launch): vehicles and receivers on side streams, the merged
-  // tree on the caller's stream, joined before the update returns
+                                             s->tx_vel, s->bbox, s->frame_trees, together);
+  const bool rebuild = s->n_updates % s->rebuild_every == 0;
+  if (together) {
+    CK(frame_trees_build(s->frame_trees, s->dyn, s->rxb, s->mix, s->veh_lo, s->veh_hi, s->V,
+                         rebuild, s->rx_pos, n_rx, st));
+    if (s->V && !rebuild) CK(bvh_refit_boxes(s->dyn, s->veh_lo, s->veh_hi, st));
+    s->n_updates++;
+    s->updated = true;
+    CK(cudaGetLastError());
+    return EMRT_OK;
+  }
+  // larger frames: the three trees are independent builds, vehicles and
+  // receivers on side streams, the merged tree on the caller's stream, joined
+  // before the update returns
   CK(cudaEventRecord(s->ev_fork, st));
   for (int k = 0; k < 2; k++) CK(cudaStreamWaitEvent(s->side[k], s->ev_fork, 0));
   if (s->V) {
-    if (s->n_updates % s->rebuild_every == 0)
+    if (rebuild)
       CK(bvh_build_boxes(s->dyn, s->veh_lo, s->veh_hi, s->V, s->bbox, s->hist_side[0], s->side[0]));
     else
       CK(bvh_refit_boxes(s->dyn, s->veh_lo, s->veh_hi, s->side[0]));
   }
   CK(bvh_build_points(s->rxb, s->rx_pos, n_rx, s->bbox, s->hist_side[1], s->side[1]));
   // vehicles and receivers in one tree for discovery's per-segment query
-  const uint32_t nm = s->V + n_rx;
   emrt::note_launch(), k_mix_prims<<<ceil_div(nm, 256), 256, 0, st>>>(s->veh_lo, s->veh_hi, s->V,
                                                                      s->rx_pos, n_rx, s->mix_lo,
                                                                      s->mix_hi);

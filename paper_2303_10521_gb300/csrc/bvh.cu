@@ -7,40 +7,11 @@
 #include <cuda/atomic>
 
 #include "bvh.cuh"
+#include "lbvh.cuh"
 
 namespace emrt {
 
 namespace {
-
-__device__ inline uint64_t spread3(uint32_t v) {
-  uint64_t x = v & 0x1fffffu;
-  x = (x | x << 32) & 0x1f00000000ffffull;
-  x = (x | x << 16) & 0x1f0000ff0000ffull;
-  x = (x | x << 8) & 0x100f00f00f00f00full;
-  x = (x | x << 4) & 0x10c30c30c30c30c3ull;
-  x = (x | x << 2) & 0x1249249249249249ull;
-  return x;
-}
-
-// Morton code (3 AB bits, AB <= 21 per axis) of p quantised in the cube
-// spanned by the largest extent of the box (all axes share one scale), so
-// that a flat scene is split along its long axes first instead of slicing it
-// into thin horizontal slabs.  Equal codes are told apart by index in the
-// hierarchy (delta), so coarse codes only cost tree quality.
-template <int AB>
-__device__ inline uint64_t morton_code(float3 p, const float4 *bb) {
-  float4 lo = bb[0], hi = bb[1];
-  float ext = fmaxf(fmaxf(hi.x - lo.x, hi.y - lo.y), fmaxf(hi.z - lo.z, 1e-6f));
-  float q[3] = {(p.x - lo.x) / ext, (p.y - lo.y) / ext, (p.z - lo.z) / ext};
-  uint32_t c[3];
-  for (int k = 0; k < 3; k++)
-    c[k] = (uint32_t)(fminf(fmaxf(q[k], 0.f), 1.f) * (float)((1u << AB) - 1u));
-  return spread3(c[0]) << 2 | spread3(c[1]) << 1 | spread3(c[2]);
-}
-// code bits per primitive kind: the static triangles (LBVH fallback) use 63;
-// vehicle boxes and receiver points, rebuilt every frame, use 30 (2 m cells
-// over a 2 km cube) so that their sort takes four passes instead of eight
-constexpr int kMortonBitsTri = 21, kMortonBitsDyn = 10;
 
 __device__ inline void put_key(KeyW<2> &k, uint64_t v) {
   k.w[0] = (uint32_t)v;
@@ -77,46 +48,6 @@ __global__ void k_morton_points(const float4 *p, uint32_t n, const float4 *bb, K
   if (i >= n) return;
   put_key(keys[i], morton_code<kMortonBitsDyn>(f3(p[i]), bb));
   idx[i] = i;
-}
-
-// Inner node i in [0, n-2] of the radix tree over the sorted keys k: its
-// range, split and children, and the parent links of the children.
-template <typename KeyAt>
-__device__ inline void hierarchy_node(KeyAt key, int n, int i, float4 *nodes,
-                                      uint32_t *leaf_parent) {
-  auto delta = [&](int a, int c) -> int {
-    if (c < 0 || c >= n) return -1;
-    const uint64_t x = key(a), y = key(c);
-    if (x == y) return 64 + __clz(a ^ c);
-    return __clzll(x ^ y);
-  };
-  int d = (delta(i, i + 1) - delta(i, i - 1)) >= 0 ? 1 : -1;
-  int dmin = delta(i, i - d);
-  int lmax = 2;
-  while (delta(i, i + lmax * d) > dmin) lmax <<= 1;
-  int l = 0;
-  for (int t = lmax >> 1; t >= 1; t >>= 1)
-    if (delta(i, i + (l + t) * d) > dmin) l += t;
-  int j = i + l * d;
-  int dnode = delta(i, j);
-  int s = 0, t = l;
-  do {
-    t = (t + 1) >> 1;
-    if (delta(i, i + (s + t) * d) > dnode) s += t;
-  } while (t > 1);
-  int gamma = i + s * d + min(d, 0);
-  int left = min(i, j) == gamma ? ~gamma : gamma;
-  int right = max(i, j) == gamma + 1 ? ~(gamma + 1) : gamma + 1;
-  int *n3 = reinterpret_cast<int *>(nodes + 4ll * i + 3);
-  n3[0] = left;
-  n3[1] = right;
-  n3[3] = 0;
-  int code0 = 2 * i, code1 = 2 * i + 1;
-  if (left < 0) leaf_parent[~left] = code0;
-  else reinterpret_cast<int *>(nodes + 4ll * left + 3)[2] = code0;
-  if (right < 0) leaf_parent[~right] = code1;
-  else reinterpret_cast<int *>(nodes + 4ll * right + 3)[2] = code1;
-  if (i == 0) n3[2] = -1;
 }
 
 // one thread per inner node i in [0, n-2]

@@ -70,6 +70,32 @@ cudaError_t bvh_refit_boxes(BVHBuf &b, const float4 *lo, const float4 *hi, cudaS
 // on the node's grid.  Synchronises the stream (build time only).
 cudaError_t bvh8_build(BVHBuf &b, cudaStream_t s);
 
+// Scratch of frame_trees_build (owned by the scene).
+struct FrameTreesBuf {
+  uint32_t *count = nullptr;   // [2 kTreeBins] primitives, vehicles of a bin
+  uint32_t *code = nullptr;    // [2 cap] Morton codes of the frame's primitives
+                               // (vehicles, then receivers), places in their bins
+  uint32_t *first = nullptr;   // [2 (kTreeBins + 1)] positions of the bins
+  uint2 *member = nullptr;     // [cap] the bins' lists
+  uint32_t *sorted = nullptr;  // codes of the three trees in order
+  float4 *blocks = nullptr;    // boxes of aligned blocks of leaves
+  uint32_t cap = 0;
+};
+// Bins of the leading 12 of a code's 30 bits (125 m cells over a 2 km cube).
+constexpr uint32_t kTreeBins = 4096, kTreeBinShift = 18;
+// Primitives (vehicles + receivers) up to which the per-frame trees are built
+// together: the codes of the widest tree have to fit a block's shared memory
+// (128 KB here); at 32760 the update takes 54 us against 126 us.
+constexpr uint32_t kFrameTreesMax = 32768;
+cudaError_t frame_trees_alloc(FrameTreesBuf &b, uint32_t n);
+void frame_trees_free(FrameTreesBuf &b);
+// Builds the receiver tree, the merged tree and, when `vehicles`, the vehicle
+// tree of a frame of V + R <= min(f.cap, kFrameTreesMax) primitives whose
+// codes, places and bin counts are at f (see frame_code in lbvh.cuh).
+cudaError_t frame_trees_build(const FrameTreesBuf &f, BVHBuf &veh, BVHBuf &rx, BVHBuf &mix,
+                              const float4 *veh_lo, const float4 *veh_hi, uint32_t V,
+                              bool vehicles, const float4 *rx_pos, uint32_t R, cudaStream_t s);
+
 // Runs the per-frame builds' grid barrier once in a cooperative launch of 4
 // blocks expecting 4 + missing arrivals (synchronous): passed = blocks that
 // got through, timed_out = 1 when a block gave up (ERR_WAIT).

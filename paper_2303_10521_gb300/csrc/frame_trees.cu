@@ -1,0 +1,382 @@
+// The three per-frame trees (vehicles, receivers, both merged) of up to
+// kFrameTreesMax primitives, built together in four launches.  Same trees as
+// the one-block, cooperative and device-wide builders of bvh.cu: the order by
+// (Morton code, index), the radix tree over it, and boxes that are exact
+// minima and maxima.
+//
+// At these sizes a build is a chain of latencies, not of work, so the steps
+// are chosen to have none that wait on one another:
+//  - The sorted position of a primitive is its bin's first position (bins of
+//    the code's leading bits, counted while the codes are made) plus the
+//    smaller keys of the bin, counted directly (k_tree_bins, k_tree_rank),
+//    instead of sort passes with a barrier each.  One bin list serves all
+//    three trees: the order of the merged tree, restricted to a class, is
+//    that class's own.
+//  - A node's box is the minimum and maximum over its range of leaves, read
+//    from the aligned power-of-two blocks of k_tree_blocks, instead of a walk
+//    from the leaves up with one atomic arrival per level.
+// Measured, update replayed from a graph, against one-block (to 4096
+// primitives) and cooperative builds on three streams: 1200 primitives 61 ->
+// 29 us, 4000 124 -> 31, 15000 (the city) 109 -> 37, 32760 126 -> 54.
+#include "bvh.cuh"
+#include "lbvh.cuh"
+
+namespace emrt {
+
+namespace {
+
+struct FrameTreesView {
+  const float4 *veh_lo, *veh_hi, *rx;
+  uint32_t V, R;                // vehicles, receivers: primitives 0..V-1, V..V+R-1
+  const uint32_t *code, *slot;  // [V + R] Morton codes and places within their bins
+  const uint32_t *count, *count_v;  // [kTreeBins] primitives, vehicles
+  uint32_t *first, *first_v;    // [kTreeBins + 1] the same before a bin
+  uint2 *member;                // [V + R] (code, primitive), bin by bin
+  float4 *prims[3];             // leaves in order: vehicles (may be null), receivers, merged
+  uint32_t *sorted[3];          // their codes in order
+};
+
+// Every block scans the bins' counts (8 bins a thread) and puts its own
+// primitives into the bins' lists; block 0 keeps the scan for k_tree_rank.
+constexpr int kBinsBlock = 512, kBinsPer = kTreeBins / kBinsBlock;
+static_assert(kBinsPer == 8, "two 16-byte loads of each count a thread");
+__global__ void __launch_bounds__(kBinsBlock) k_tree_bins(FrameTreesView T) {
+  __shared__ uint32_t s_first[kTreeBins];
+  __shared__ uint2 s_warp[kBinsBlock / 32];
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t c[kBinsPer], v[kBinsPer], sc = 0, sv = 0;
+#pragma unroll
+  for (int q = 0; q < kBinsPer / 4; q++) {
+    const uint4 x = reinterpret_cast<const uint4 *>(T.count)[threadIdx.x * (kBinsPer / 4) + q];
+    const uint4 y = reinterpret_cast<const uint4 *>(T.count_v)[threadIdx.x * (kBinsPer / 4) + q];
+    c[4 * q] = x.x; c[4 * q + 1] = x.y; c[4 * q + 2] = x.z; c[4 * q + 3] = x.w;
+    v[4 * q] = y.x; v[4 * q + 1] = y.y; v[4 * q + 2] = y.z; v[4 * q + 3] = y.w;
+  }
+#pragma unroll
+  for (int q = 0; q < kBinsPer; q++) {
+    sc += c[q];
+    sv += v[q];
+  }
+  uint32_t ic = sc, iv = sv;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t a = __shfl_up_sync(0xffffffffu, ic, o), b = __shfl_up_sync(0xffffffffu, iv, o);
+    if (lane >= (uint32_t)o) {
+      ic += a;
+      iv += b;
+    }
+  }
+  if (lane == 31) s_warp[warp] = make_uint2(ic, iv);
+  __syncthreads();
+  uint32_t bc = ic - sc, bv = iv - sv;
+  for (uint32_t w = 0; w < warp; w++) {
+    bc += s_warp[w].x;
+    bv += s_warp[w].y;
+  }
+#pragma unroll
+  for (int q = 0; q < kBinsPer; q++) {
+    const uint32_t bin = threadIdx.x * kBinsPer + q;
+    s_first[bin] = bc;
+    if (blockIdx.x == 0) {
+      T.first[bin] = bc;
+      T.first_v[bin] = bv;
+    }
+    bc += c[q];
+    bv += v[q];
+  }
+  if (blockIdx.x == 0 && threadIdx.x == kBinsBlock - 1) {
+    T.first[kTreeBins] = bc;
+    T.first_v[kTreeBins] = bv;
+  }
+  __syncthreads();
+  const uint32_t p = blockIdx.x * kBinsBlock + threadIdx.x;
+  if (p >= T.V + T.R) return;
+  const uint32_t code = T.code[p];
+  T.member[s_first[code >> kTreeBinShift] + T.slot[p]] = make_uint2(code, p);
+}
+
+// One thread a list place (a warp's threads mostly share their bin, whose
+// list they read together): smaller keys of the bin, of both classes and of
+// its own, and the leaf written in its places.
+constexpr int kRankBlock = 128;
+__global__ void __launch_bounds__(kRankBlock) k_tree_rank(FrameTreesView T) {
+  const uint32_t i = blockIdx.x * kRankBlock + threadIdx.x;
+  if (i >= T.V + T.R) return;
+  const uint2 me = T.member[i];
+  const uint32_t p = me.y, bin = me.x >> kTreeBinShift;
+  const bool veh = p < T.V;
+  const uint32_t b0 = T.first[bin], b1 = T.first[bin + 1], v0 = T.first_v[bin];
+  const float4 a = veh ? T.veh_lo[p] : T.rx[p - T.V], b = veh ? T.veh_hi[p] : a;
+  uint32_t mix = 0, vehs = 0;
+#pragma unroll 4
+  for (uint32_t q = b0; q < b1; q++) {
+    const uint2 m = T.member[q];
+    const bool less = m.x < me.x || (m.x == me.x && m.y < p);  // equal codes by index
+    mix += less ? 1u : 0u;
+    vehs += less && m.y < T.V ? 1u : 0u;
+  }
+  const uint32_t own = veh ? v0 + vehs : b0 - v0 + mix - vehs;
+  mix += b0;
+  T.prims[2][2ull * mix] = make_float4(a.x, a.y, a.z, __uint_as_float(p));
+  T.prims[2][2ull * mix + 1] = make_float4(b.x, b.y, b.z, 0.f);
+  T.sorted[2][mix] = me.x;
+  if (!veh) {
+    T.prims[1][own] = make_float4(a.x, a.y, a.z, __uint_as_float(p - T.V));
+    T.sorted[1][own] = me.x;
+  } else if (T.prims[0]) {
+    T.prims[0][2ull * own] = make_float4(a.x, a.y, a.z, __uint_as_float(p));
+    T.prims[0][2ull * own + 1] = make_float4(b.x, b.y, b.z, 0.f);
+    T.sorted[0][own] = me.x;
+  }
+}
+
+// Boxes of aligned blocks of leaves: level l (1..kLevels) has ceil(n / 2^l)
+// of them, two float4 (lo, hi) each, one level after the other.
+constexpr int kLevels = 10;
+constexpr int kBlocksBlock = 256;
+constexpr uint32_t kBlocksLeaves = 1u << kLevels;  // leaves of a thread block
+
+struct TreeView {       // one tree of the last two launches
+  const float4 *prims;
+  const uint32_t *sorted;
+  float4 *blocks;
+  float4 *nodes;
+  uint32_t *leaf_parent;
+  uint32_t n;
+  uint32_t first;       // first thread block of the launch that serves it
+  int points;           // 1: leaves are points (one float4), 0: boxes (two)
+};
+struct TreeSet {
+  TreeView t[3];
+};
+
+struct LoHi {
+  float3 lo, hi;
+};
+// Merging ignores NaN (fminf, fmaxf), so NaN is the box of nothing.
+__device__ inline LoHi no_box() {
+  const float q = __int_as_float(0x7fffffff);
+  return LoHi{make_float3(q, q, q), make_float3(q, q, q)};
+}
+__device__ inline void merge(LoHi &a, const LoHi &b) {
+  a.lo = make_float3(fminf(a.lo.x, b.lo.x), fminf(a.lo.y, b.lo.y), fminf(a.lo.z, b.lo.z));
+  a.hi = make_float3(fmaxf(a.hi.x, b.hi.x), fmaxf(a.hi.y, b.hi.y), fmaxf(a.hi.z, b.hi.z));
+}
+__device__ inline LoHi leaf_of(const TreeView &t, uint32_t g) {
+  LoHi b;
+  if (t.points) {
+    b.lo = b.hi = f3(t.prims[g]);
+  } else {
+    b.lo = f3(t.prims[2ull * g]);
+    b.hi = f3(t.prims[2ull * g + 1]);
+  }
+  return b;
+}
+__device__ inline void put_block(const TreeView &t, uint32_t offset, int level, uint32_t i,
+                                 const LoHi &b) {
+  if (((uint64_t)i << level) >= t.n) return;
+  t.blocks[2ull * (offset + i)] = make_float4(b.lo.x, b.lo.y, b.lo.z, 0.f);
+  t.blocks[2ull * (offset + i) + 1] = make_float4(b.hi.x, b.hi.y, b.hi.z, 0.f);
+}
+__device__ inline LoHi shfl_box(const LoHi &b, int d) {
+  LoHi r;
+  r.lo = make_float3(__shfl_down_sync(0xffffffffu, b.lo.x, d), __shfl_down_sync(0xffffffffu, b.lo.y, d),
+                     __shfl_down_sync(0xffffffffu, b.lo.z, d));
+  r.hi = make_float3(__shfl_down_sync(0xffffffffu, b.hi.x, d), __shfl_down_sync(0xffffffffu, b.hi.y, d),
+                     __shfl_down_sync(0xffffffffu, b.hi.z, d));
+  return r;
+}
+// the tree a thread block of the launch serves (no dynamic indexing of the
+// kernel's parameters)
+__device__ inline TreeView tree_of(const TreeSet &S) {
+  TreeView t = S.t[0];
+  if (blockIdx.x >= S.t[1].first) t = S.t[1];
+  if (blockIdx.x >= S.t[2].first) t = S.t[2];
+  return t;
+}
+
+// Four leaves a thread (levels 1 and 2), a warp's 32 by shuffles (3-7), the
+// block's eight warps by shuffles of the first (8-10): no step waits for
+// another block.
+__global__ void __launch_bounds__(kBlocksBlock) k_tree_blocks(TreeSet S) {
+  __shared__ LoHi s_warp[kBlocksBlock / 32];
+  const TreeView t = tree_of(S);
+  const uint32_t base = (blockIdx.x - t.first) * kBlocksLeaves;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t g = base + 4u * threadIdx.x;
+  LoHi b[4];
+#pragma unroll
+  for (int q = 0; q < 4; q++) b[q] = g + q < t.n ? leaf_of(t, g + q) : no_box();
+  merge(b[0], b[1]);
+  merge(b[2], b[3]);
+  uint32_t offset = 0;
+  put_block(t, offset, 1, g / 2, b[0]);
+  put_block(t, offset, 1, g / 2 + 1, b[2]);
+  merge(b[0], b[2]);
+  offset += (t.n + 1) >> 1;
+  put_block(t, offset, 2, g / 4, b[0]);
+  for (int l = 3; l <= 7; l++) {
+    offset += (t.n + (1u << (l - 1)) - 1) >> (l - 1);
+    const int d = 1 << (l - 3);
+    merge(b[0], shfl_box(b[0], d));
+    if ((lane & (2 * d - 1)) == 0) put_block(t, offset, l, g >> l, b[0]);
+  }
+  if (lane == 0) s_warp[warp] = b[0];
+  __syncthreads();
+  if (warp) return;
+  b[0] = lane < kBlocksBlock / 32 ? s_warp[lane] : no_box();
+  for (int l = 8; l <= kLevels; l++) {
+    offset += (t.n + (1u << (l - 1)) - 1) >> (l - 1);
+    const int d = 1 << (l - 8);
+    merge(b[0], shfl_box(b[0], d));
+    if (lane < kBlocksBlock / 32 && (lane & (2 * d - 1)) == 0)
+      put_block(t, offset, l, (base >> l) + (lane >> (l - 7)), b[0]);
+  }
+}
+
+// Boxes of leaves first..split and split + 1..last: the aligned blocks they
+// are made of, at most two a level each and the run of the top level.  Both
+// ranges go up the levels together and a level's loads are issued before its
+// merges: the loads' latency is the time of this step.
+__device__ inline void range_boxes(const TreeView &t, const NodeRange &r, LoHi &a, LoHi &b) {
+  a = b = no_box();
+  uint32_t l0 = r.first, r0 = r.split + 1, l1 = r.split + 1, r1 = r.last + 1, offset = 0;
+  for (int level = 0; l0 < r0 || l1 < r1; level++) {
+    auto at = [&](bool take, uint32_t i) {
+      if (!take) return no_box();
+      if (level == 0) return leaf_of(t, i);
+      return LoHi{f3(t.blocks[2ull * (offset + i)]), f3(t.blocks[2ull * (offset + i) + 1])};
+    };
+    if (level == kLevels) {
+      for (; l0 < r0; l0++) merge(a, at(true, l0));
+      for (; l1 < r1; l1++) merge(b, at(true, l1));
+      break;
+    }
+    const bool la = l0 < r0 && (l0 & 1u), ra = l0 + la < r0 && (r0 & 1u);
+    const bool lb = l1 < r1 && (l1 & 1u), rb = l1 + lb < r1 && (r1 & 1u);
+    const LoHi x = at(la, l0), y = at(ra, r0 - 1), z = at(lb, l1), w = at(rb, r1 - 1);
+    merge(a, x);
+    merge(a, y);
+    merge(b, z);
+    merge(b, w);
+    l0 = (l0 + 1) >> 1;
+    r0 >>= 1;
+    l1 = (l1 + 1) >> 1;
+    r1 >>= 1;
+    if (level > 0) offset += (t.n + (1u << level) - 1) >> level;
+  }
+}
+
+// One thread an inner node: its range and split from the codes in shared
+// memory, then the boxes of its two children.
+constexpr int kNodesBlock = 256;
+__global__ void __launch_bounds__(kNodesBlock) k_tree_nodes(TreeSet S, float pad) {
+  extern __shared__ __align__(16) uint32_t s_codes[];
+  const TreeView t = tree_of(S);
+  {  // the tree's codes, 16 bytes at a time (arrays start and end on 16 bytes)
+    const uint4 *in = reinterpret_cast<const uint4 *>(t.sorted);
+    uint4 *out = reinterpret_cast<uint4 *>(s_codes);
+#pragma unroll 4
+    for (uint32_t k = threadIdx.x; k < (t.n + 3) / 4; k += kNodesBlock) out[k] = in[k];
+  }
+  __syncthreads();
+  const uint32_t i = (blockIdx.x - t.first) * kNodesBlock + threadIdx.x;
+  if (i + 1 >= t.n) return;
+  const NodeRange r = hierarchy_node([](int q) { return s_codes[q]; }, (int)t.n, (int)i,
+                                     t.nodes, t.leaf_parent);
+  LoHi a, b;
+  range_boxes(t, r, a, b);
+  float4 *n = t.nodes + 4ull * i;
+  n[0] = make_float4(a.lo.x - pad, a.hi.x + pad, a.lo.y - pad, a.hi.y + pad);
+  n[1] = make_float4(b.lo.x - pad, b.hi.x + pad, b.lo.y - pad, b.hi.y + pad);
+  n[2] = make_float4(a.lo.z - pad, a.hi.z + pad, b.lo.z - pad, b.hi.z + pad);
+}
+
+}  // namespace
+
+static uint32_t round4(uint32_t n) { return (n + 3u) & ~3u; }
+
+cudaError_t frame_trees_alloc(FrameTreesBuf &b, uint32_t n) {
+  frame_trees_free(b);
+  if (n > kFrameTreesMax) n = kFrameTreesMax;  // larger frames take the other builders
+  b.cap = n;
+  // counts; codes, slots; first positions; member lists
+  cudaError_t e = cudaMalloc((void **)&b.count, sizeof(uint32_t) * 2 * kTreeBins);
+  if (!e) e = cudaMalloc((void **)&b.code, sizeof(uint32_t) * 2ull * n);
+  if (!e) e = cudaMalloc((void **)&b.first, sizeof(uint32_t) * 2 * (kTreeBins + 1));
+  if (!e) e = cudaMalloc((void **)&b.member, sizeof(uint2) * n);
+  // sorted codes and block boxes (below n + kLevels a tree) of the three trees
+  if (!e) e = cudaMalloc((void **)&b.sorted, sizeof(uint32_t) * (2ull * n + 12));
+  if (!e) e = cudaMalloc((void **)&b.blocks, 2 * sizeof(float4) * (2ull * n + 3ull * (kLevels + 1)));
+  return e;
+}
+
+void frame_trees_free(FrameTreesBuf &b) {
+  cudaFree(b.count);
+  cudaFree(b.code);
+  cudaFree(b.first);
+  cudaFree(b.member);
+  cudaFree(b.sorted);
+  cudaFree(b.blocks);
+  b = FrameTreesBuf{};
+}
+
+cudaError_t frame_trees_build(const FrameTreesBuf &f, BVHBuf &veh, BVHBuf &rx, BVHBuf &mix,
+                              const float4 *veh_lo, const float4 *veh_hi, uint32_t V,
+                              bool vehicles, const float4 *rx_pos, uint32_t R, cudaStream_t s) {
+  const uint32_t n = V + R;
+  FrameTreesView T{};
+  T.veh_lo = veh_lo;
+  T.veh_hi = veh_hi;
+  T.rx = rx_pos;
+  T.V = V;
+  T.R = R;
+  T.code = f.code;
+  T.slot = f.code + f.cap;
+  T.count = f.count;
+  T.count_v = f.count + kTreeBins;
+  T.first = f.first;
+  T.first_v = f.first + kTreeBins + 1;
+  T.member = f.member;
+  T.prims[0] = vehicles ? veh.prims : nullptr;
+  T.prims[1] = rx.prims;
+  T.prims[2] = mix.prims;
+  T.sorted[2] = f.sorted;
+  T.sorted[0] = f.sorted + round4(n);
+  T.sorted[1] = T.sorted[0] + round4(V);
+  if (vehicles) veh.n = V;
+  rx.n = R;
+  mix.n = n;
+  emrt::note_launch(), k_tree_bins<<<ceil_div(n, kBinsBlock), kBinsBlock, 0, s>>>(T);
+  emrt::note_launch(), k_tree_rank<<<ceil_div(n, kRankBlock), kRankBlock, 0, s>>>(T);
+  TreeSet S{};
+  BVHBuf *buf[3] = {&veh, &rx, &mix};
+  float4 *blocks = f.blocks;
+  uint32_t nodes_first[3], blocks_total = 0, nodes_total = 0, widest = 0;
+  for (int k = 0; k < 3; k++) {
+    TreeView &t = S.t[k];
+    t.n = k == 0 ? (vehicles ? V : 0u) : k == 1 ? R : n;
+    t.prims = buf[k]->prims;
+    t.sorted = T.sorted[k];
+    t.nodes = buf[k]->nodes;
+    t.leaf_parent = buf[k]->leaf_parent;
+    t.points = k == 1;
+    t.blocks = blocks;
+    t.first = blocks_total;
+    nodes_first[k] = nodes_total;
+    if (t.n < 2) t.n = 0;  // no inner node
+    blocks += 2ull * (t.n + kLevels + 1);
+    blocks_total += ceil_div(t.n, kBlocksLeaves);
+    nodes_total += ceil_div(t.n, kNodesBlock);
+    if (t.n > widest) widest = t.n;
+  }
+  if (!nodes_total) return cudaGetLastError();
+  emrt::note_launch(), k_tree_blocks<<<blocks_total, kBlocksBlock, 0, s>>>(S);
+  for (int k = 0; k < 3; k++) S.t[k].first = nodes_first[k];
+  const size_t smem = sizeof(uint32_t) * round4(widest);
+  if (smem > 48 * 1024)
+    cudaFuncSetAttribute(k_tree_nodes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  emrt::note_launch(), k_tree_nodes<<<nodes_total, kNodesBlock, smem, s>>>(S, mix.pad);
+  return cudaGetLastError();
+}
+
+}  // namespace emrt

@@ -17,7 +17,8 @@ struct emrt_scene_s {
   BVHBuf stat, dyn, rxb;
   BVHBuf txb;                     // transmitter points (backward tracing)
   BVHBuf mix;                     // vehicles + receivers (merged per-frame tree)
-  float4 *mix_lo = nullptr, *mix_hi = nullptr;  // its primitive corners
+  float4 *mix_lo = nullptr, *mix_hi = nullptr;  // its primitive corners (large frames)
+  FrameTreesBuf frame_trees;      // scratch of the per-frame builds
   float4 *src_pos = nullptr;      // receiver points shot from (backward tracing)
   uint64_t src_cap = 0;
   float4 *veh_half = nullptr, *veh_lo = nullptr, *veh_hi = nullptr, *veh_vel = nullptr;
