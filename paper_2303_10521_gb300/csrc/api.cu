@@ -113,13 +113,7 @@ __global__ void k_mix_prims(const float4 *vlo, const float4 *vhi, uint32_t V, co
   }
 }
 
-__global__ void k_check_cand(Counters *c, uint32_t cap) {
-  if (c->n_cand > cap) atomicOr(&c->err, ERR_CAND_OVERFLOW);
-}
-
 __global__ void k_publish_count(const Counters *c, uint32_t *count) { *count = c->n_accepted; }
-
-__global__ void k_clamp_count(const uint32_t *n, uint32_t cap, uint32_t *out) { *out = min(*n, cap); }
 
 // records removed by the last revalidation: entered - kept
 __global__ void k_evicted(const Counters *c, uint32_t *out) { *out = c->n_eff - c->n_accepted; }
@@ -146,24 +140,16 @@ cudaError_t ensure_cand(emrt_scene_s *s, uint64_t need) {
   return cudaSuccess;
 }
 
-// Sort + unique of records [0, *n) of `src` (capacity cap) into s->uniq;
-// unique count in ctr->n_unique.
-void dedup(emrt_scene_s *s, const uint32_t *src, const uint32_t *n, uint32_t cap, KeyLayout kl,
-           cudaStream_t st) {
-  Counters *c = s->ctr;
-  launch_path_keys(src, n, cap, kl, s->keys[0], s->vals[0], &c->n_eff, st);
-  // radix passes over the top kDedupPasses bytes only; the runs equal there
-  // (a few candidates each) are then sorted in place by the whole key
-  const int passes = (kl.total + 7) / 8;
-  const int first = passes > kDedupPasses + 1 ? passes - kDedupPasses : 0;
-  bool alt = radix_sort<4>(&c->n_eff, s->keys[0], s->vals[0], s->keys[1], s->vals[1], kl.total,
-                           s->hist, st, cap, first);
-  KeyW<4> *ks = s->keys[alt ? 1 : 0];
-  uint32_t *vs = s->vals[alt ? 1 : 0];
-  if (first) launch_sort_runs(ks, vs, &c->n_eff, 8 * first, st);
-  launch_heads(ks, &c->n_eff, s->head, st);
-  exclusive_scan(&c->n_eff, s->head, s->pos, &c->n_unique, s->partial, st);
-  launch_unique(src, ks, vs, s->head, s->pos, &c->n_eff, s->uniq, st);
+// The pair counts, for n pairs (zeroed by each trace).
+cudaError_t ensure_pairs(emrt_scene_s *s, uint64_t n) {
+  if (n <= s->pair_cap && s->pair_count) return cudaSuccess;
+  uint64_t c = 0;
+  cudaError_t e;
+  s->pair_cap = 0;
+  e = grow(&s->pair_count, c, pair_words(n)); if (e) return e; c = 0;
+  e = grow(&s->pair_off, c, n + 4); if (e) return e;
+  s->pair_cap = n;
+  return cudaSuccess;
 }
 
 emrt_status check_paths(const emrt_paths *p) {
@@ -320,8 +306,7 @@ void emrt_scene_destroy(emrt_scene s) {
     if (s->ev_side[k]) cudaEventDestroy(s->ev_side[k]);
   }
   if (s->ev_fork) cudaEventDestroy(s->ev_fork);
-  cudaFree(s->rv_rec); cudaFree(s->rv_head); cudaFree(s->rv_pos); cudaFree(s->rv_partial);
-  cudaFree(s->rv_apts); cudaFree(s->rv_ctr);
+  cudaFree(s->rv_rec); cudaFree(s->rv_partial); cudaFree(s->rv_apts); cudaFree(s->rv_ctr);
   for (auto &t : s->dt) {
     cudaFree(t.dirs);
     cudaFree(t.stab);
@@ -334,6 +319,7 @@ void emrt_scene_destroy(emrt_scene s) {
   for (int k = 0; k < 2; k++) { cudaFree(s->rkeys[k]); cudaFree(s->rvals[k]); }
   cudaFree(s->cand); cudaFree(s->uniq); cudaFree(s->head); cudaFree(s->pos); cudaFree(s->apts);
   for (int k = 0; k < 2; k++) { cudaFree(s->keys[k]); cudaFree(s->vals[k]); }
+  cudaFree(s->pair_count); cudaFree(s->pair_off);
   cudaFree(s->contrib);
   for (int k = 0; k < 4; k++)
     if (s->ev[k]) cudaEventDestroy(s->ev[k]);
@@ -416,35 +402,26 @@ int id_bits(uint64_t v) {
 // canonical dedup, image-method acceptance in the scene's forward geometry
 // and compaction into out.  count: rays per source; jbits: ray-index bits of
 // the ray ids.
-// Revalidation of cache on stream st with the scratch (rec, head, pos,
-// partial, apts; capacity cap >= cache->capacity) and counters c.
+// Revalidation of cache on stream st with the scratch (rec, partial, apts;
+// capacity cap >= cache->capacity) and counters c.
 void revalidate_with(emrt_scene_s *s, emrt_paths *cache, uint32_t flags, cudaStream_t st,
-                     uint32_t *rec, uint32_t *head, uint32_t *pos, uint32_t *partial,
-                     float4 *apts, uint32_t cap, Counters *c) {
+                     uint32_t *rec, uint32_t *partial, float4 *apts, uint32_t cap, Counters *c) {
   GeomView g = geom(s);
-  // clamp the count to the capacity before acceptance
-  emrt::note_launch(), k_clamp_count<<<1, 1, 0, st>>>(cache->count, cache->capacity, &c->n_eff);
-  launch_copy_records(cache->rec, &c->n_eff, rec, cache->capacity, st);
+  launch_copy_paths(cache->rec, cache->count, cache->capacity, rec, &c->n_eff, st);
   launch_accept(g, rec, &c->n_eff, c, apts, cap, st);
-  int keep_all = (flags & EMRT_REVALIDATE_KEEP) ? 1 : 0;
-  launch_keep_flags(rec, &c->n_eff, keep_all, head, st);
-  exclusive_scan(&c->n_eff, head, pos, &c->n_accepted, partial, st);
-  launch_scatter(rec, &c->n_eff, head, pos, cache->rec, cache->capacity, &c->n_accepted, c, st);
-  emrt::note_launch(), k_publish_count<<<1, 1, 0, st>>>(c, cache->count);
+  launch_keep(rec, &c->n_eff, (flags & EMRT_REVALIDATE_KEEP) ? KEEP_ALL : KEEP_VALID, cache->rec,
+              cache->capacity, nullptr, &c->n_accepted, cache->count, c, partial, st);
 }
 
 // The side-stream revalidation scratch, sized for cap records.
 cudaError_t ensure_rv(emrt_scene_s *s, uint64_t cap) {
   if (cap <= s->rv_cap && s->rv_rec) return cudaSuccess;
-  cudaFree(s->rv_rec); cudaFree(s->rv_head); cudaFree(s->rv_pos); cudaFree(s->rv_partial);
-  cudaFree(s->rv_apts);
-  s->rv_rec = s->rv_head = s->rv_pos = s->rv_partial = nullptr;
+  cudaFree(s->rv_rec); cudaFree(s->rv_partial); cudaFree(s->rv_apts);
+  s->rv_rec = s->rv_partial = nullptr;
   s->rv_apts = nullptr;
   s->rv_cap = 0;
   cudaError_t e;
   if ((e = cudaMalloc(&s->rv_rec, sizeof(uint32_t) * 8 * cap))) return e;
-  if ((e = cudaMalloc(&s->rv_head, sizeof(uint32_t) * cap))) return e;
-  if ((e = cudaMalloc(&s->rv_pos, sizeof(uint32_t) * cap))) return e;
   if ((e = cudaMalloc(&s->rv_partial, sizeof(uint32_t) * (kPrimGrid + 1)))) return e;
   if ((e = cudaMalloc(&s->rv_apts, sizeof(float4) * (EMRT_MAX_DEPTH + 2) * cap))) return e;
   if (!s->rv_ctr && (e = cudaMalloc(&s->rv_ctr, sizeof(Counters)))) return e;
@@ -452,33 +429,19 @@ cudaError_t ensure_rv(emrt_scene_s *s, uint64_t cap) {
   return cudaSuccess;
 }
 
-// main counters <- error bits and occlusion rays of the side revalidation
-__global__ void k_fold_counters(const Counters *side, Counters *c) {
-  atomicOr(&c->err, side->err);
-  c->occl_rays += side->occl_rays;
-}
-
-// Tail of a rediscovery: the unique candidates in s->uniq (count n_unique,
-// canonical) that the cache does not hold are accepted, and the accepted
-// ones merged into the cache (both canonical and disjoint: a merge-path
-// gather, no duplicate runs).
-void rediscover_tail(emrt_scene_s *s, const GeomView &g, emrt_paths *cache, cudaStream_t st) {
+// Tail of a rediscovery: the ordered candidates in s->cand (count n_eff) that
+// the cache does not hold are accepted, and the accepted ones merged into the
+// cache (both canonical and disjoint).  side: counters of the cache's
+// revalidation on another stream (may be null).
+void rediscover_tail(emrt_scene_s *s, const GeomView &g, emrt_paths *cache, const Counters *side,
+                     cudaStream_t st) {
   Counters *c = s->ctr;
-  const KeyLayout kl = key_layout(s->n_tx, s->n_rx, s->Fs + 6 * s->V + 1, EMRT_MAX_DEPTH);
-  launch_known(s->uniq, &c->n_unique, cache->rec, cache->count, cache->capacity, kl, s->head, st);
-  exclusive_scan(&c->n_unique, s->head, s->pos, &c->n_eff, s->partial, st);
-  launch_scatter(s->uniq, &c->n_unique, s->head, s->pos, s->cand, s->cand_cap, &c->n_eff, c, st);
+  launch_known(s->cand, &c->n_eff, cache->rec, cache->count, cache->capacity, side, c, st);
   launch_accept(g, s->cand, &c->n_eff, c, s->apts, s->cand_cap, st);
-  launch_keep_flags(s->cand, &c->n_eff, 0, s->head, st);
-  exclusive_scan(&c->n_eff, s->head, s->pos, &c->tmp, s->partial, st);
-  launch_scatter(s->cand, &c->n_eff, s->head, s->pos, s->uniq, s->cand_cap, &c->tmp, c, st);
-  launch_concat(cache->rec, cache->count, cache->capacity, s->uniq, &c->tmp, s->cand_cap, s->cand,
-                s->cand_cap, &c->n_accepted, c, st);
-  launch_path_keys(s->cand, &c->n_accepted, s->cand_cap, kl, s->keys[0], s->vals[0], &c->n_eff, st);
-  launch_merge_path(s->keys[0], s->vals[0], cache->count, cache->capacity, &c->n_eff, s->keys[1],
-                    s->vals[1], c, st);
-  launch_gather_records(s->cand, s->vals[1], &c->n_eff, cache->rec, cache->capacity, c, st);
-  emrt::note_launch(), k_clamp_count<<<1, 1, 0, st>>>(&c->n_eff, 0xffffffffu, cache->count);
+  launch_keep(s->cand, &c->n_eff, KEEP_VALID, s->uniq, s->cand_cap, nullptr, &c->tmp, nullptr, c,
+              s->partial, st);
+  launch_merge_paths(cache->rec, cache->count, cache->capacity, s->uniq, &c->tmp, s->cand,
+                     s->cand_cap, c, st);
 }
 
 emrt_status run_trace(emrt_scene_s *s, const emrt_trace_params *p, uint64_t count,
@@ -486,8 +449,8 @@ emrt_status run_trace(emrt_scene_s *s, const emrt_trace_params *p, uint64_t coun
                       const uint32_t *rx_ids, emrt_paths *out, cudaStream_t st,
                       emrt_paths *merge_cache = nullptr, cudaEvent_t merge_after = nullptr) {
   uint32_t nf = s->Fs + 6 * s->V;
-  KeyLayout kl = key_layout(s->n_tx, s->n_rx, nf + 1, (int)p->max_depth);
-  if (kl.total > 128) return EMRT_ERR_INVALID_ARG;
+  if (key_layout(s->n_tx, s->n_rx, nf + 1, (int)p->max_depth).total > 128)
+    return EMRT_ERR_INVALID_ARG;
   Counters *c = s->ctr;
   // primary direction table of this ray set (built once, kept in an LRU of 4)
   emrt_scene_s::DirTable *tab = nullptr;
@@ -573,6 +536,9 @@ emrt_status run_trace(emrt_scene_s *s, const emrt_trace_params *p, uint64_t coun
   // candidate scratch
   want = merge_cache ? want + out->capacity : std::max<uint64_t>(want, out->capacity);
   CK(ensure_cand(s, want));
+  const uint32_t n_pairs = s->n_tx * s->n_rx;
+  CK(ensure_pairs(s, n_pairs));
+  cudaMemsetAsync(s->pair_count, 0, sizeof(uint32_t) * pair_words(n_pairs), st);
   // counters: keep the error word, clear the rest
   cudaMemsetAsync(reinterpret_cast<char *>(c) + sizeof(uint32_t), 0,
                   sizeof(Counters) - sizeof(uint32_t), st);
@@ -670,28 +636,19 @@ emrt_status run_trace(emrt_scene_s *s, const emrt_trace_params *p, uint64_t coun
   }
   s->ev_bounces = nev;
   cudaEventRecord(s->ev[1], st);
-  emrt::note_launch(), k_check_cand<<<1, 1, 0, st>>>(c, s->cand_cap);
   if (backward) launch_reverse_candidates(s->cand, &c->n_cand, s->cand_cap, rx_ids, st);
-  dedup(s, s->cand, &c->n_cand, s->cand_cap, kl, st);
+  launch_dedup(s->cand, &c->n_cand, s->cand_cap, PairSpace{nullptr, s->n_rx, n_pairs},
+               pair_bufs(s->pair_count, s->pair_off, n_pairs), s->uniq, s->pos, c, s->partial, st);
   cudaEventRecord(s->ev[2], st);
   if (merge_cache) {
-    if (merge_after) {  // the cache's revalidation on the side stream
+    if (merge_after)  // the cache's revalidation on the side stream
       CK(cudaStreamWaitEvent(st, merge_after, 0));
-      emrt::note_launch(), k_fold_counters<<<1, 1, 0, st>>>(s->rv_ctr, c);
-    }
-    rediscover_tail(s, g, merge_cache, st);
-    cudaEventRecord(s->ev[3], st);
-    s->ev_recorded = true;
-    CK(cudaGetLastError());
-    return EMRT_OK;
+    rediscover_tail(s, g, merge_cache, merge_after ? s->rv_ctr : nullptr, st);
+  } else {
+    launch_accept(g, s->cand, &c->n_eff, c, s->apts, s->cand_cap, st);
+    launch_keep(s->cand, &c->n_eff, (p->flags & EMRT_TRACE_KEEP_REJECTED) ? KEEP_PATHS : KEEP_VALID,
+                out->rec, out->capacity, nullptr, &c->n_accepted, out->count, c, s->partial, st);
   }
-  launch_accept(g, s->uniq, &c->n_unique, c, s->apts, s->cand_cap, st);
-  launch_keep_flags(s->uniq, &c->n_unique, (p->flags & EMRT_TRACE_KEEP_REJECTED) ? 1 : 0, s->head,
-                    st);
-  exclusive_scan(&c->n_unique, s->head, s->pos, &c->n_accepted, s->partial, st);
-  launch_scatter(s->uniq, &c->n_unique, s->head, s->pos, out->rec, out->capacity, &c->n_accepted,
-                 c, st);
-  emrt::note_launch(), k_publish_count<<<1, 1, 0, st>>>(c, out->count);
   cudaEventRecord(s->ev[3], st);
   s->ev_recorded = true;
   CK(cudaGetLastError());
@@ -743,8 +700,8 @@ emrt_status emrt_rediscover(emrt_scene s, const emrt_trace_params *p, emrt_paths
     CK(cudaEventRecord(s->ev_fork, st));
     CK(cudaStreamWaitEvent(s->side[0], s->ev_fork, 0));
     cudaMemsetAsync(s->rv_ctr, 0, sizeof(Counters), s->side[0]);
-    revalidate_with(s, cache, 0u, s->side[0], s->rv_rec, s->rv_head, s->rv_pos, s->rv_partial,
-                    s->rv_apts, (uint32_t)s->rv_cap, s->rv_ctr);
+    revalidate_with(s, cache, 0u, s->side[0], s->rv_rec, s->rv_partial, s->rv_apts,
+                    (uint32_t)s->rv_cap, s->rv_ctr);
     CK(cudaEventRecord(s->ev_side[0], s->side[0]));
     after = s->ev_side[0];
   }
@@ -789,8 +746,7 @@ emrt_status emrt_revalidate(emrt_scene s, emrt_paths *cache, uint32_t flags, emr
   if (!s->updated) return EMRT_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
   CK(ensure_cand(s, std::max<uint64_t>(s->want_cand, cache->capacity)));
-  revalidate_with(s, cache, flags, st, s->uniq, s->head, s->pos, s->partial, s->apts, s->cand_cap,
-                  s->ctr);
+  revalidate_with(s, cache, flags, st, s->uniq, s->partial, s->apts, s->cand_cap, s->ctr);
   CK(cudaGetLastError());
   return EMRT_OK;
 }

@@ -34,14 +34,12 @@ struct emrt_batch_s {
   KeyW<1> *rkeys[2] = {nullptr, nullptr};
   uint32_t *rvals[2] = {nullptr, nullptr};
   uint32_t cand_cap = 0, want_cand = 0;
-  uint32_t *cand = nullptr, *uniq = nullptr, *head = nullptr, *pos = nullptr;
+  uint32_t *cand = nullptr, *uniq = nullptr, *pos = nullptr;
   float4 *apts = nullptr;  // acceptance scratch (reflection points)
-  KeyW<4> *keys[2] = {nullptr, nullptr};
-  uint32_t *vals[2] = {nullptr, nullptr};
-  uint32_t *first = nullptr, *cnt = nullptr;
+  uint32_t *pair_count = nullptr, *pair_off = nullptr;  // candidates of every (scene, tx, rx)
+  uint32_t n_pairs = 0;
   Counters *ctr = nullptr;
   uint32_t *hist = nullptr, *partial = nullptr;
-  KeyLayout kl{};
   int variant = default_bounce_variant();
   bool sort_rays = false;
   uint32_t largest = 0;  // scene whose box quantises the ray sort keys
@@ -65,12 +63,9 @@ emrt_status st_of(cudaError_t e) {
   } while (0)
 
 void free_scratch(emrt_batch_s *b) {
-  cudaFree(b->cand); cudaFree(b->uniq); cudaFree(b->head); cudaFree(b->pos); cudaFree(b->apts);
-  for (int k = 0; k < 2; k++) { cudaFree(b->keys[k]); cudaFree(b->vals[k]); }
-  b->cand = b->uniq = b->head = b->pos = nullptr;
+  cudaFree(b->cand); cudaFree(b->uniq); cudaFree(b->pos); cudaFree(b->apts);
+  b->cand = b->uniq = b->pos = nullptr;
   b->apts = nullptr;
-  b->keys[0] = b->keys[1] = nullptr;
-  b->vals[0] = b->vals[1] = nullptr;
   b->cand_cap = 0;
 }
 
@@ -80,13 +75,8 @@ cudaError_t alloc_cand(emrt_batch_s *b, uint64_t cap) {
   cudaError_t e;
   if ((e = cudaMalloc(&b->cand, 32 * cap))) return e;
   if ((e = cudaMalloc(&b->uniq, 32 * cap))) return e;
-  if ((e = cudaMalloc(&b->head, 4 * cap))) return e;
   if ((e = cudaMalloc(&b->pos, 4 * cap))) return e;
   if ((e = cudaMalloc(&b->apts, sizeof(float4) * (EMRT_MAX_DEPTH + 2) * cap))) return e;
-  for (int k = 0; k < 2; k++) {
-    if ((e = cudaMalloc(&b->keys[k], sizeof(KeyW<4>) * cap))) return e;
-    if ((e = cudaMalloc(&b->vals[k], 4 * cap))) return e;
-  }
   b->cand_cap = (uint32_t)cap;
   return cudaSuccess;
 }
@@ -124,7 +114,7 @@ void drop_graph(emrt_batch_s *b) {
 
 // current per-scene table (host side, pinned)
 void fill_table(emrt_batch_s *b) {
-  uint32_t begin = 0;
+  uint32_t begin = 0, pairs = 0;
   for (uint32_t i = 0; i < b->n; i++) {
     emrt_scene s = b->scenes[i];
     BatchScene &t = b->h_tab[i];
@@ -140,6 +130,9 @@ void fill_table(emrt_batch_s *b) {
     t.out_rec = b->outs[i].rec;
     t.out_cap = b->outs[i].capacity;
     t.out_count = b->outs[i].count;
+    t.pair_begin = pairs;
+    t.pair_rx = s->max_rx;
+    pairs += b->n_tx[i] * s->max_rx;
   }
 }
 
@@ -176,23 +169,16 @@ void enqueue(emrt_batch_s *b, int variant, bool sort_rays, cudaStream_t st) {
     L.K = (int)b->Kmax;
     launch_bounce_batched(variant, L, b->d_tab, b->n, st);
   }
-  // deduplicate (keys carry the scene), accept, scatter to each scene
-  launch_path_keys(b->cand, &c->n_cand, b->cand_cap, b->kl, b->keys[0], b->vals[0], &c->n_eff, st);
-  const int passes = (b->kl.total + 7) / 8;
-  const int first = passes > kDedupPasses + 1 ? passes - kDedupPasses : 0;
-  bool alt = radix_sort<4>(&c->n_eff, b->keys[0], b->vals[0], b->keys[1], b->vals[1], b->kl.total,
-                           b->hist, st, b->cand_cap, first);
-  KeyW<4> *ks = b->keys[alt ? 1 : 0];
-  uint32_t *vs = b->vals[alt ? 1 : 0];
-  if (first) launch_sort_runs(ks, vs, &c->n_eff, 8 * first, st);
-  launch_heads(ks, &c->n_eff, b->head, st);
-  exclusive_scan(&c->n_eff, b->head, b->pos, &c->n_unique, b->partial, st);
-  launch_unique(b->cand, ks, vs, b->head, b->pos, &c->n_eff, b->uniq, st);
-  launch_accept_batched(b->d_tab, b->uniq, &c->n_unique, c, b->apts, b->cand_cap, st);
-  launch_keep_flags(b->uniq, &c->n_unique, 0, b->head, st);
-  exclusive_scan(&c->n_unique, b->head, b->pos, &c->n_accepted, b->partial, st);
-  launch_batch_scatter(b->d_tab, b->n, b->uniq, &c->n_unique, b->head, b->pos, b->first, b->cnt,
-                       c, st);
+  // canonical order (records carry the scene), accept, write to each scene
+  const PairSpace ps{b->d_tab, 0, b->n_pairs};
+  cudaMemsetAsync(b->pair_count, 0, sizeof(uint32_t) * pair_words(b->n_pairs), st);
+  const PairBufs pairs = pair_bufs(b->pair_count, b->pair_off, b->n_pairs);
+  launch_dedup(b->cand, &c->n_cand, b->cand_cap, ps, pairs, b->uniq, b->pos, c, b->partial, st);
+  launch_accept_batched(b->d_tab, b->cand, &c->n_eff, c, b->apts, b->cand_cap, st);
+  launch_keep(b->cand, &c->n_eff, KEEP_VALID, nullptr, 0, b->pos, &c->n_accepted, nullptr, c,
+              b->partial, st);
+  launch_batch_write(b->d_tab, b->n, b->cand, &c->n_eff, pairs.off, b->n_pairs, b->pos,
+                     &c->n_accepted, c, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -257,7 +243,7 @@ emrt_status emrt_batch_create(const emrt_scene *scenes, uint32_t n, const emrt_t
   };
   b->n = n;
   uint32_t max_rx = 1, max_tx = 1, max_f = 1;
-  uint64_t tris = 0;
+  uint64_t tris = 0, n_pairs = 0;
   for (uint32_t i = 0; i < n; i++) {
     emrt_scene s = scenes[i];
     const emrt_trace_params &p = params[i];
@@ -277,6 +263,7 @@ emrt_status emrt_batch_create(const emrt_scene *scenes, uint32_t n, const emrt_t
     b->n_tx.push_back(s->n_tx);
     b->total += count * s->n_tx;
     b->Kmax = std::max(b->Kmax, p.max_depth);
+    n_pairs += (uint64_t)s->n_tx * s->max_rx;
     max_rx = std::max(max_rx, s->max_rx);
     max_tx = std::max(max_tx, s->n_tx);
     max_f = std::max(max_f, s->Fs + 6 * s->V + 1);
@@ -284,15 +271,15 @@ emrt_status emrt_batch_create(const emrt_scene *scenes, uint32_t n, const emrt_t
     tris += s->T;
   }
   if (b->total >= (1ull << 32)) return fail(EMRT_ERR_INVALID_ARG);
-  b->kl = key_layout(max_tx, max_rx, max_f, (int)b->Kmax, n);
-  if (b->kl.total > 128) return fail(EMRT_ERR_INVALID_ARG);
+  if (key_layout(max_tx, max_rx, max_f, (int)b->Kmax, n).total > 128) return fail(EMRT_ERR_INVALID_ARG);
   BCK(cudaMallocHost(&b->h_tab, sizeof(BatchScene) * n));
   BCK(cudaMalloc(&b->d_tab, sizeof(BatchScene) * n));
   BCK(cudaMalloc(&b->ctr, sizeof(Counters)));
   BCK(cudaMalloc(&b->hist, sizeof(uint32_t) * (256 * kPrimGrid + 1)));
   BCK(cudaMalloc(&b->partial, sizeof(uint32_t) * (kPrimGrid + 1)));
-  BCK(cudaMalloc(&b->first, sizeof(uint32_t) * kBatchMaxScenes));
-  BCK(cudaMalloc(&b->cnt, sizeof(uint32_t) * kBatchMaxScenes));
+  b->n_pairs = (uint32_t)n_pairs;
+  BCK(cudaMalloc(&b->pair_count, sizeof(uint32_t) * pair_words(n_pairs)));
+  BCK(cudaMalloc(&b->pair_off, sizeof(uint32_t) * (n_pairs + 4)));
   BCK(cudaMemsetAsync(b->ctr, 0, sizeof(Counters), st));
   // direction tables, shared between scenes with the same ray set
   KeyW<1> *k0 = nullptr;
@@ -477,7 +464,7 @@ void emrt_batch_destroy(emrt_batch b) {
   free_rays(b);
   for (auto p : b->owned_dirs) cudaFree(p);
   cudaFree(b->d_tab); cudaFree(b->ctr); cudaFree(b->hist); cudaFree(b->partial);
-  cudaFree(b->first); cudaFree(b->cnt);
+  cudaFree(b->pair_count); cudaFree(b->pair_off);
   if (b->h_tab) cudaFreeHost(b->h_tab);
   delete b;
 }

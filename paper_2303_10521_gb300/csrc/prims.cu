@@ -75,30 +75,6 @@ __global__ void __launch_bounds__(1024) k_digit_offsets(const uint32_t *d_n, uin
   }
 }
 
-// exclusive scan of n (<= a few 100k) words in one block of 1024 threads
-__global__ void __launch_bounds__(1024) k_scan_single(uint32_t *v, uint32_t n, uint32_t *total) {
-  __shared__ uint32_t part[1024];
-  uint32_t per = (n + 1023) / 1024;
-  uint32_t lo = min(n, threadIdx.x * per), hi = min(n, lo + per);
-  uint32_t s = 0;
-  for (uint32_t i = lo; i < hi; i++) s += v[i];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int off = 1; off < 1024; off <<= 1) {
-    uint32_t t = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
-    __syncthreads();
-    part[threadIdx.x] += t;
-    __syncthreads();
-  }
-  uint32_t run = part[threadIdx.x] - s;
-  for (uint32_t i = lo; i < hi; i++) {
-    uint32_t t = v[i];
-    v[i] = run;
-    run += t;
-  }
-  if (threadIdx.x == 1023 && total) *total = part[1023];
-}
-
 // Stable scatter of one radix pass.  The block's key range (block_range) is
 // processed in tiles of kPrimBlock * IPT keys held in registers; warp w owns
 // tile elements [w * 32 * IPT, (w + 1) * 32 * IPT), its lane l the elements
@@ -229,14 +205,33 @@ __global__ void __launch_bounds__(kPrimBlock) k_scan_reduce(const uint32_t *d_n,
   }
 }
 
+// Every block sums the partial sums before its own (at most kPrimGrid words)
+// instead of a launch that scans them.
 __global__ void __launch_bounds__(kPrimBlock) k_scan_down(const uint32_t *d_n, const uint32_t *in,
-                                                          uint32_t *out, const uint32_t *partial) {
+                                                          uint32_t *out, const uint32_t *partial,
+                                                          uint32_t *total) {
   __shared__ uint32_t sh[kPrimBlock / 32];
-  __shared__ uint32_t carry;
+  __shared__ uint32_t carry, all;
   uint32_t lo, hi;
   block_range(*d_n, lo, hi);
-  if (threadIdx.x == 0) carry = partial[blockIdx.x];
+  if (threadIdx.x == 0) carry = all = 0;
   __syncthreads();
+  uint32_t mine = 0, every = 0;
+  for (uint32_t b = threadIdx.x; b < gridDim.x; b += kPrimBlock) {
+    const uint32_t c = partial[b];
+    every += c;
+    mine += b < blockIdx.x ? c : 0u;
+  }
+  for (int o = 16; o; o >>= 1) {
+    mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    every += __shfl_xor_sync(0xffffffffu, every, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&carry, mine);
+    atomicAdd(&all, every);
+  }
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && total) *total = all;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (uint32_t r0 = lo; r0 < hi; r0 += kPrimBlock) {
     uint32_t i = r0 + threadIdx.x;
@@ -276,7 +271,7 @@ bool radix_sort(const uint32_t *d_n, KeyW<W> *keys, uint32_t *vals, KeyW<W> *key
     uint32_t *vi = alt ? vals2 : vals, *vo = alt ? vals : vals2;
     emrt::note_launch(), k_hist<W><<<G, kPrimBlock, 0, s>>>(d_n, ki, p, hist);
     emrt::note_launch(), k_digit_offsets<<<1, 1024, 0, s>>>(d_n, hist, G);
-    emrt::note_launch(), k_scatter<W, (W == 4 ? 4 : 8)><<<G, kPrimBlock, 0, s>>>(d_n, ki, vi, ko, vo, p, hist);
+    emrt::note_launch(), k_scatter<W, 8><<<G, kPrimBlock, 0, s>>>(d_n, ki, vi, ko, vo, p, hist);
     alt = !alt;
   }
   return alt;
@@ -286,14 +281,10 @@ template bool radix_sort<1>(const uint32_t *, KeyW<1> *, uint32_t *, KeyW<1> *, 
                             int, uint32_t *, cudaStream_t, uint64_t, int);
 template bool radix_sort<2>(const uint32_t *, KeyW<2> *, uint32_t *, KeyW<2> *, uint32_t *,
                             int, uint32_t *, cudaStream_t, uint64_t, int);
-template bool radix_sort<4>(const uint32_t *, KeyW<4> *, uint32_t *, KeyW<4> *, uint32_t *,
-                            int, uint32_t *, cudaStream_t, uint64_t, int);
-
 void exclusive_scan(const uint32_t *d_n, const uint32_t *in, uint32_t *out, uint32_t *d_total,
                     uint32_t *partial, cudaStream_t s) {
   emrt::note_launch(), k_scan_reduce<<<kPrimGrid, kPrimBlock, 0, s>>>(d_n, in, partial);
-  emrt::note_launch(), k_scan_single<<<1, 1024, 0, s>>>(partial, kPrimGrid, d_total);
-  emrt::note_launch(), k_scan_down<<<kPrimGrid, kPrimBlock, 0, s>>>(d_n, in, out, partial);
+  emrt::note_launch(), k_scan_down<<<kPrimGrid, kPrimBlock, 0, s>>>(d_n, in, out, partial, d_total);
 }
 
 }  // namespace emrt

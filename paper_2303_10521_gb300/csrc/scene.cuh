@@ -57,15 +57,18 @@ struct emrt_scene_s {
   float4 *apts = nullptr;  // acceptance scratch: reflection points, point-major
   KeyW<4> *keys[2] = {nullptr, nullptr};
   uint32_t *vals[2] = {nullptr, nullptr};
+  // candidates of every (tx, rx) pair: counts and places (max_tx x max_rx)
+  uint32_t *pair_count = nullptr, *pair_off = nullptr;
+  uint64_t pair_cap = 0;
   // adjoint scratch
   double *contrib = nullptr;
   uint64_t contrib_cap = 0;
   emrt_status sticky = EMRT_OK;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   // revalidation scratch of a rediscovery that revalidates its cache on a
-  // side stream while the discovery runs: records, flags, positions, scan
-  // partials, reflection points (capacity rv_cap) and its own counters
-  uint32_t *rv_rec = nullptr, *rv_head = nullptr, *rv_pos = nullptr, *rv_partial = nullptr;
+  // side stream while the discovery runs: records, block counts, reflection
+  // points (capacity rv_cap) and its own counters
+  uint32_t *rv_rec = nullptr, *rv_partial = nullptr;
   float4 *rv_apts = nullptr;
   Counters *rv_ctr = nullptr;
   uint64_t rv_cap = 0;

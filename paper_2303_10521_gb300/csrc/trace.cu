@@ -177,111 +177,6 @@ __global__ void k_merge_path(const KeyW<4> *keys, const uint32_t *vals, const ui
   }
 }
 
-// equal keys above bit lb
-__device__ inline bool key_prefix_eq(const KeyW<4> &a, const KeyW<4> &b, int lb) {
-#pragma unroll
-  for (int q = 0; q < 4; q++) {
-    const int lo = 32 * q;
-    if (lo + 32 <= lb) continue;
-    const int sh = lb > lo ? lb - lo : 0;
-    if ((a.w[q] >> sh) != (b.w[q] >> sh)) return false;
-  }
-  return true;
-}
-
-// Completes a sort ordered by the key bits from lb up: each run of keys equal
-// in those bits is sorted by the whole key, in place, by the thread at its
-// head (insertion sort for short runs, heap sort for long ones; the order of
-// equal keys is not kept).
-__global__ void k_sort_runs(KeyW<4> *k, uint32_t *v, const uint32_t *n, int lb) {
-  const uint32_t cnt = *n;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
-    if (i > 0 && key_prefix_eq(k[i], k[i - 1], lb)) continue;
-    uint32_t e = i + 1;
-    while (e < cnt && key_prefix_eq(k[e], k[i], lb)) e++;
-    const uint32_t len = e - i;
-    if (len < 2) continue;
-    KeyW<4> *kk = k + i;
-    uint32_t *vv = v + i;
-    if (len <= 32) {
-      for (uint32_t a = 1; a < len; a++) {
-        const KeyW<4> x = kk[a];
-        const uint32_t xv = vv[a];
-        uint32_t b = a;
-        while (b > 0 && key_lt(x, kk[b - 1])) {
-          kk[b] = kk[b - 1];
-          vv[b] = vv[b - 1];
-          b--;
-        }
-        kk[b] = x;
-        vv[b] = xv;
-      }
-      continue;
-    }
-    auto swap = [&](uint32_t a, uint32_t b) {
-      const KeyW<4> t = kk[a];
-      kk[a] = kk[b];
-      kk[b] = t;
-      const uint32_t tv = vv[a];
-      vv[a] = vv[b];
-      vv[b] = tv;
-    };
-    auto sift = [&](uint32_t root, uint32_t end) {
-      while (2 * root + 1 < end) {
-        uint32_t c = 2 * root + 1;
-        if (c + 1 < end && key_lt(kk[c], kk[c + 1])) c++;
-        if (!key_lt(kk[root], kk[c])) break;
-        swap(root, c);
-        root = c;
-      }
-    };
-    for (uint32_t r = len / 2; r-- > 0;) sift(r, len);
-    for (uint32_t end = len - 1; end > 0; end--) {
-      swap(0, end);
-      sift(0, end);
-    }
-  }
-}
-
-// Candidates already in the cache: for each of the *n unique candidates (in
-// canonical order) a binary search of the cache's canonical records;
-// flag[i] = 1 for a candidate the cache does not hold.  A candidate the
-// cache holds as a valid path lowers that record's smallest ray index to its
-// own (what merging the accepted candidate would have done; one candidate per
-// record, so no two threads write the same word).
-__global__ void k_known(const uint32_t *cand, const uint32_t *n, uint32_t *cache,
-                        const uint32_t *cache_n, uint32_t cache_cap, KeyLayout kl,
-                        uint32_t *flag) {
-  const uint32_t cnt = *n, nc = min(*cache_n, cache_cap);
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
-    const KeyW<4> k = record_key(cand + 8ull * i, kl);
-    uint32_t lo = 0, hi = nc;
-    while (lo < hi) {  // first cache record whose key is not below k
-      const uint32_t mid = (lo + hi) >> 1;
-      if (key_lt(record_key(cache + 8ull * mid, kl), k)) lo = mid + 1;
-      else hi = mid;
-    }
-    const bool found = lo < nc && key_eq(record_key(cache + 8ull * lo, kl), k);
-    flag[i] = found ? 0u : 1u;
-    if (found && (cache[8ull * lo + 2] & EMRT_PATH_VALID))
-      cache[8ull * lo + 7] = min(cache[8ull * lo + 7], cand[8ull * i + 7]);
-  }
-}
-
-// out[k] = rec[vals[k]] for k < min(*n, cap); ERR_PATH_OVERFLOW when *n > cap.
-__global__ void k_gather_records(const uint32_t *rec, const uint32_t *vals, const uint32_t *n,
-                                 uint32_t *out, uint32_t cap, Counters *ctr) {
-  const uint32_t cnt = *n;
-  uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0 && cnt > cap) atomicOr(&ctr->err, ERR_PATH_OVERFLOW);
-  for (; i < min(cnt, cap); i += gridDim.x * blockDim.x) {
-    const uint4 *r = reinterpret_cast<const uint4 *>(rec + 8ull * vals[i]);
-    uint4 *o = reinterpret_cast<uint4 *>(out + 8ull * i);
-    o[0] = r[0];
-    o[1] = r[1];
-  }
-}
-
 __global__ void k_heads(const KeyW<4> *keys, const uint32_t *n, uint32_t *head) {
   uint32_t cnt = *n;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x)
@@ -498,16 +393,6 @@ __global__ void k_scatter_rec(const uint32_t *in, const uint32_t *n, const uint3
   }
 }
 
-__global__ void k_copy_rec(const uint32_t *in, const uint32_t *n, uint32_t *out, uint32_t cap) {
-  uint32_t cnt = min(*n, cap);
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
-    const uint4 *s = reinterpret_cast<const uint4 *>(in + 8ull * i);
-    uint4 *d = reinterpret_cast<uint4 *>(out + 8ull * i);
-    d[0] = s[0];
-    d[1] = s[1];
-  }
-}
-
 __global__ void k_concat(const uint32_t *a, const uint32_t *na, uint32_t cap_a, const uint32_t *b,
                          const uint32_t *nb, uint32_t cap_b, uint32_t *dst, uint32_t dst_cap,
                          uint32_t *n_dst, Counters *ctr) {
@@ -547,50 +432,6 @@ __global__ void k_reverse_cand(uint32_t *cand, const uint32_t *n, uint32_t cap,
       r[k] = (uint32_t)k < depth ? f[depth - 1 - k] : EMRT_NO_FACE;
     c[0] = make_uint4(a.y, ids ? ids[a.x] : a.x, a.z, r[0]);
     c[1] = make_uint4(r[1], r[2], r[3], b.w);
-  }
-}
-
-__global__ void k_batch_first(const uint32_t *rec, const uint32_t *n, const uint32_t *flag,
-                              const uint32_t *pos, uint32_t *first, uint32_t *cnt) {
-  uint32_t c = *n;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < c; i += gridDim.x * blockDim.x) {
-    if (!flag[i]) continue;
-    uint32_t sc = rec[8ull * i] >> 8;
-    if (sc >= kBatchMaxScenes) continue;
-    atomicMin(&first[sc], pos[i]);
-    atomicAdd(&cnt[sc], 1u);
-  }
-}
-
-__global__ void k_batch_write(const BatchScene *tab, uint32_t n_scenes, const uint32_t *rec,
-                              const uint32_t *n, const uint32_t *flag, const uint32_t *pos,
-                              const uint32_t *first, const uint32_t *cnt, Counters *ctr) {
-  uint32_t c = *n;
-  uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n_scenes) {
-    *tab[t].out_count = cnt[t];
-    if (cnt[t] > tab[t].out_cap) atomicOr(&ctr->err, ERR_PATH_OVERFLOW);
-  }
-  for (uint32_t i = t; i < c; i += gridDim.x * blockDim.x) {
-    if (!flag[i]) continue;
-    const uint4 *src = reinterpret_cast<const uint4 *>(rec + 8ull * i);
-    uint4 a = src[0], b = src[1];
-    uint32_t sc = a.x >> 8;
-    if (sc >= n_scenes) continue;
-    uint32_t p = pos[i] - first[sc];
-    if (p >= tab[sc].out_cap) continue;
-    a.x &= 255u;
-    uint4 *dst = reinterpret_cast<uint4 *>(tab[sc].out_rec + 8ull * p);
-    dst[0] = a;
-    dst[1] = b;
-  }
-}
-
-__global__ void k_batch_init(uint32_t *first, uint32_t *cnt) {
-  uint32_t t = threadIdx.x;
-  if (t < kBatchMaxScenes) {
-    first[t] = 0xffffffffu;
-    cnt[t] = 0u;
   }
 }
 
@@ -747,15 +588,6 @@ void launch_accept_batched(const BatchScene *tab, uint32_t *rec, const uint32_t 
   emrt::note_launch(), k_accept_occl<true><<<kPrimGrid * 8, kBounceBlock, 0, s>>>(none, tab, rec, n, pts, cap, ctr);
 }
 
-void launch_batch_scatter(const BatchScene *tab, uint32_t n_scenes, const uint32_t *rec,
-                          const uint32_t *n, const uint32_t *flag, const uint32_t *pos,
-                          uint32_t *first, uint32_t *cnt, Counters *ctr, cudaStream_t s) {
-  emrt::note_launch(), k_batch_init<<<1, kBatchMaxScenes, 0, s>>>(first, cnt);
-  emrt::note_launch(), k_batch_first<<<kPrimGrid * 4, 256, 0, s>>>(rec, n, flag, pos, first, cnt);
-  emrt::note_launch(), k_batch_write<<<kPrimGrid * 4, 256, 0, s>>>(tab, n_scenes, rec, n, flag, pos,
-                                                                  first, cnt, ctr);
-}
-
 void build_dir_table(uint64_t n_rays, uint64_t offset, uint64_t stride, uint32_t count,
                      float4 *table, KeyW<1> *k0, KeyW<1> *k1, uint32_t *v0, uint32_t *v1,
                      uint32_t *d_n, uint32_t *hist, cudaStream_t s) {
@@ -805,10 +637,6 @@ void launch_scatter(const uint32_t *in, const uint32_t *n, const uint32_t *flag,
                     Counters *ctr, cudaStream_t s) {
   emrt::note_launch(), k_scatter_rec<<<kPrimGrid * 4, 256, 0, s>>>(in, n, flag, pos, out, cap, total, ctr);
 }
-void launch_copy_records(const uint32_t *in, const uint32_t *n, uint32_t *out, uint32_t cap,
-                         cudaStream_t s) {
-  emrt::note_launch(), k_copy_rec<<<kPrimGrid * 4, 256, 0, s>>>(in, n, out, cap);
-}
 void launch_concat(const uint32_t *a, const uint32_t *na, uint32_t cap_a, const uint32_t *b,
                    const uint32_t *nb, uint32_t cap_b, uint32_t *dst, uint32_t dst_cap,
                    uint32_t *n_dst, Counters *ctr, cudaStream_t s) {
@@ -818,18 +646,6 @@ void launch_merge_path(const KeyW<4> *keys, const uint32_t *vals, const uint32_t
                        const uint32_t *n, KeyW<4> *kout, uint32_t *vout, Counters *ctr,
                        cudaStream_t s) {
   emrt::note_launch(), k_merge_path<<<kPrimGrid * 4, 256, 0, s>>>(keys, vals, na, cap_a, n, kout, vout, ctr);
-}
-void launch_known(const uint32_t *cand, const uint32_t *n, uint32_t *cache, const uint32_t *cache_n,
-                  uint32_t cache_cap, KeyLayout kl, uint32_t *flag, cudaStream_t s) {
-  emrt::note_launch(), k_known<<<kPrimGrid * 4, 256, 0, s>>>(cand, n, cache, cache_n, cache_cap, kl, flag);
-}
-void launch_gather_records(const uint32_t *rec, const uint32_t *vals, const uint32_t *n,
-                           uint32_t *out, uint32_t cap, Counters *ctr, cudaStream_t s) {
-  emrt::note_launch(), k_gather_records<<<kPrimGrid * 4, 256, 0, s>>>(rec, vals, n, out, cap, ctr);
-}
-void launch_sort_runs(KeyW<4> *keys, uint32_t *vals, const uint32_t *n, int low_bits,
-                      cudaStream_t s) {
-  emrt::note_launch(), k_sort_runs<<<kPrimGrid * 4, 256, 0, s>>>(keys, vals, n, low_bits);
 }
 void launch_set_u32(uint32_t *p, uint32_t v, cudaStream_t s) { emrt::note_launch(), k_set_u32<<<1, 1, 0, s>>>(p, v); }
 

@@ -86,6 +86,8 @@ struct BatchScene {
   uint32_t *out_rec;      // caller's output records
   uint32_t out_cap;
   uint32_t *out_count;
+  uint32_t pair_begin;    // first pair of this scene in the batch's pair space
+  uint32_t pair_rx;       // its receiver capacity (pairs of a transmitter)
 };
 constexpr uint32_t kBatchMaxScenes = 64, kBatchMaxTx = 16, kBatchMaxCount = 1u << 22;
 
@@ -104,13 +106,6 @@ void launch_bounce_batched(int variant, const BounceLaunch &L, const BatchScene 
 // records [0, min(*n, cap))
 void launch_accept_batched(const BatchScene *tab, uint32_t *rec, const uint32_t *n, Counters *ctr,
                            float4 *pts, uint32_t cap, cudaStream_t s);
-// writes kept, sorted batched records to each scene's output (positions
-// relative to the scene's first kept record); first[] and cnt[] are
-// kBatchMaxScenes words of scratch
-void launch_batch_scatter(const BatchScene *tab, uint32_t n_scenes, const uint32_t *rec,
-                          const uint32_t *n, const uint32_t *flag, const uint32_t *pos,
-                          uint32_t *first, uint32_t *cnt, Counters *ctr, cudaStream_t s);
-
 // Coherence keys of the *n rays (24 bits, three radix passes): origin cell
 // (5-bit Morton per axis in the scene box) then direction bin (9 bits of the
 // octahedral code).
@@ -140,9 +135,6 @@ void launch_keep_flags(const uint32_t *rec, const uint32_t *n, int keep_all, uin
 void launch_scatter(const uint32_t *in, const uint32_t *n, const uint32_t *flag,
                     const uint32_t *pos, uint32_t *out, uint32_t cap, const uint32_t *total,
                     Counters *ctr, cudaStream_t s);
-// out[0..min(*n,cap)) = in; *n_out = *n
-void launch_copy_records(const uint32_t *in, const uint32_t *n, uint32_t *out, uint32_t cap,
-                         cudaStream_t s);
 // concatenation of two record sets into dst (count written to *n_dst)
 void launch_concat(const uint32_t *a, const uint32_t *na, uint32_t cap_a, const uint32_t *b,
                    const uint32_t *nb, uint32_t cap_b, uint32_t *dst, uint32_t dst_cap,
@@ -153,22 +145,6 @@ void launch_concat(const uint32_t *a, const uint32_t *na, uint32_t cap_a, const 
 void launch_merge_path(const KeyW<4> *keys, const uint32_t *vals, const uint32_t *na, uint32_t cap_a,
                        const uint32_t *n, KeyW<4> *kout, uint32_t *vout, Counters *ctr,
                        cudaStream_t s);
-// flag[i] = 1 for each of the *n canonical candidate records the canonical
-// cache (min(*cache_n, cache_cap) records) does not hold; a candidate it holds
-// as a valid path lowers that record's smallest ray index (word 7).
-void launch_known(const uint32_t *cand, const uint32_t *n, uint32_t *cache, const uint32_t *cache_n,
-                  uint32_t cache_cap, KeyLayout kl, uint32_t *flag, cudaStream_t s);
-// out[k] = rec[vals[k]] for k < min(*n, cap); ERR_PATH_OVERFLOW when *n > cap.
-void launch_gather_records(const uint32_t *rec, const uint32_t *vals, const uint32_t *n,
-                           uint32_t *out, uint32_t cap, Counters *ctr, cudaStream_t s);
-// Deduplication sorts run radix passes over the top kDedupPasses bytes of
-// the canonical key only and then launch_sort_runs (measured on the city:
-// 4 passes 0.11 ms, 5 0.13, 6 0.15, all 11 0.22).
-constexpr int kDedupPasses = 4;
-// Completes a sort of (keys, vals)[0, *n) that is ordered by the key bits
-// from low_bits up: runs equal in those bits are sorted by the whole key.
-void launch_sort_runs(KeyW<4> *keys, uint32_t *vals, const uint32_t *n, int low_bits,
-                      cudaStream_t s);
 void launch_set_u32(uint32_t *p, uint32_t v, cudaStream_t s);
 
 // Backward tracing.  out[i] = pos[ids[i]] for i < n (source points of the
@@ -182,5 +158,59 @@ void launch_gather_points(const float4 *pos, const uint32_t *ids, uint32_t n, fl
 // kept.  Records [0, min(*n, cap)).
 void launch_reverse_candidates(uint32_t *cand, const uint32_t *n, uint32_t cap,
                                const uint32_t *ids, cudaStream_t s);
+
+// ---------------------------------------------------------------------------
+// Path records after discovery (paths.cu).
+// The (tx, rx) pairs candidates belong to: pair tx * n_rx + rx of one scene,
+// or the scenes' ranges of a batch's table.
+struct PairSpace {
+  const BatchScene *tab;  // null: one scene
+  uint32_t n_rx, n_pairs;
+};
+constexpr uint32_t kPairGroup = 256;  // pairs counted together once more
+struct PairBufs {
+  uint32_t *count;  // [n_pairs up to a multiple of 4], zero before a dedup, as
+  uint32_t *group;  // [n_pairs / kPairGroup rounded up]
+  uint32_t *off;    // [n_pairs + 4]
+};
+// words at count for n_pairs pairs (count, then group), and their places
+uint64_t pair_words(uint64_t n_pairs);
+PairBufs pair_bufs(uint32_t *count, uint32_t *off, uint64_t n_pairs);
+// pairs up to which a group's block sums the groups before it (4096 words)
+constexpr uint32_t kPairScanMax = 1u << 20;
+// min(*n_cand, cap) candidates at cand, in place, to canonical order; equal
+// paths become one record with the smallest ray index and duplicates behind
+// it, whose depth (word 2) is no path's.  ctr->n_eff: records, duplicates
+// included; ctr->n_unique is raised by the others (0 before).  lists, place:
+// scratch of cap records and cap words.
+void launch_dedup(uint32_t *cand, const uint32_t *n_cand, uint32_t cap, const PairSpace &ps,
+                  const PairBufs &pb, uint32_t *lists, uint32_t *place, Counters *ctr,
+                  uint32_t *partial, cudaStream_t s);
+enum KeepWhich { KEEP_VALID, KEEP_PATHS, KEEP_ALL };  // valid; not a duplicate; every record
+// The kept ones of *n records in order to out (at most cap; more raise
+// ERR_PATH_OVERFLOW), their number to *total and *count (may be null); with
+// pos, the kept records before each one instead.
+void launch_keep(const uint32_t *rec, const uint32_t *n, KeepWhich which, uint32_t *out,
+                 uint32_t cap, uint32_t *pos, uint32_t *total, uint32_t *count, Counters *ctr,
+                 uint32_t *partial, cudaStream_t s);
+// valid ones of a batch's *n ordered records to each scene's output (pos and
+// total of launch_keep, off of the batch's pairs)
+void launch_batch_write(const BatchScene *tab, uint32_t n_scenes, const uint32_t *rec,
+                        const uint32_t *n, const uint32_t *off, uint32_t n_pairs,
+                        const uint32_t *pos, const uint32_t *total, Counters *ctr,
+                        cudaStream_t s);
+// out = the *n_out = min(*count, cap) records at in
+void launch_copy_paths(const uint32_t *in, const uint32_t *count, uint32_t cap, uint32_t *out,
+                       uint32_t *n_out, cudaStream_t s);
+// Marks the *n ordered candidates that the canonical cache (min(*cache_n,
+// cache_cap) records) holds as duplicates; a candidate it holds as a valid path
+// lowers that record's smallest ray index.  side: see k_known.
+void launch_known(uint32_t *cand, const uint32_t *n, uint32_t *cache, const uint32_t *cache_n,
+                  uint32_t cache_cap, const Counters *side, Counters *ctr, cudaStream_t s);
+// cache <- cache merged with *n_new canonical records it does not hold (tmp:
+// scratch of tmp_cap records); *cache_n and ctr->n_accepted: the merged count.
+void launch_merge_paths(uint32_t *cache, uint32_t *cache_n, uint32_t cache_cap,
+                        const uint32_t *fresh, const uint32_t *n_new, uint32_t *tmp,
+                        uint32_t tmp_cap, Counters *ctr, cudaStream_t s);
 
 }  // namespace emrt
