@@ -254,6 +254,48 @@ __device__ inline double inface_margin(const GeomView &g, uint32_t f, D3 P, D3 n
 
 constexpr double kMargin = 1e-4;
 
+// inface_margin() of a reflection point P, as far as acceptance asks: whether
+// it is negative (outside the face) and whether it lies within kMargin of zero.
+// A warp issues an FP64 instruction every 64 cycles on GB300 and the margin
+// takes about 39 of them an edge, so the edges are first measured in FP32, in
+// coordinates from the face's first vertex (the difference taken in FP64):
+// with M the largest |P - a0| + |a - a0|, the FP32 distance is off by at most
+// about 13 x 2^-24 M (rounding of the three differences, of a cross and a dot
+// product and of one reciprocal root); a point whose distances all clear
+// kMargin by 2e-6 M (33 x 2^-24) on one side is decided, any other goes to the
+// FP64 margin.  Geometry of the city's 16k candidates 55 -> 24 us, of the
+// district's 3.7k 30 -> 20, of the toy scene's 38 19 -> 9.
+struct InFace {
+  bool outside, marginal;
+};
+__device__ inline InFace inface(const GeomView &g, uint32_t f, D3 P, D3 n) {
+  if (f < g.n_static_faces) {
+    const uint4 info = g.face_info[f];
+    const float3 a0 = f3(g.face_vert[info.x]);
+    const D3 p64 = P - tod(a0);
+    const float3 p = make_float3((float)p64.x, (float)p64.y, (float)p64.z);
+    const float3 nf = make_float3((float)n.x, (float)n.y, (float)n.z);
+    const float pl = fabsf(p.x) + fabsf(p.y) + fabsf(p.z);
+    float m = 1e30f, M = pl;
+    float3 a = f3(g.face_vert[info.x + info.y - 1]) - a0;
+#pragma unroll 4
+    for (uint32_t k = 0; k < info.y; k++) {
+      const float3 b = f3(g.face_vert[info.x + k]) - a0;
+      const float3 e = b - a, w = p - a;
+      const float3 c = make_float3(e.y * w.z - e.z * w.y, e.z * w.x - e.x * w.z,
+                                   e.x * w.y - e.y * w.x);
+      m = fminf(m, dot3(c, nf) * rsqrtf(dot3(e, e)));
+      M = fmaxf(M, pl + (fabsf(b.x) + fabsf(b.y) + fabsf(b.z)));
+      a = b;
+    }
+    const float slack = (float)kMargin + 2e-6f * M;
+    if (m > slack) return InFace{false, false};
+    if (m < -slack) return InFace{true, false};
+  }
+  const double m = inface_margin(g, f, P, n);
+  return InFace{m < 0.0, fabs(m) < kMargin};
+}
+
 // Acceptance runs in two phases so that the occlusion legs, long any-hit
 // traversals, get a thread each.  Phase 1, per record: images across the
 // face planes, reflection points backward from the receiver (FP64), the
@@ -302,9 +344,9 @@ __global__ void __launch_bounds__(kBounceBlock) k_accept_geom(GeomView G, const 
         double t = (dd[q - 1] - dotd(nn[q - 1], I[q])) / den;
         if (!(t > 0.0 && t < 1.0)) { ok = false; break; }
         Q[q] = I[q] + D * t;
-        double m = inface_margin(g, f[q - 1], Q[q], nn[q - 1]);
-        if (m < 0.0) ok = false;
-        if (fabs(m) < kMargin) marg = true;
+        const InFace in = inface(g, f[q - 1], Q[q], nn[q - 1]);
+        if (in.outside) ok = false;
+        if (in.marginal) marg = true;
       }
       if (ok)
         for (uint32_t q = 0; q <= k + 1; q++)
@@ -316,55 +358,102 @@ __global__ void __launch_bounds__(kBounceBlock) k_accept_geom(GeomView G, const 
   }
 }
 
-// Each leg's any-hit test is split over kOcclPieces threads, each taking
-// one piece of t in (0, 1) on the same ray (so every t is the one the whole
-// leg would compute): the leg is occluded iff some piece is.  The launch is
-// latency-bound -- a few long legs (first legs from a transmitter across
-// the city) kept most SMs idle -- and shorter pieces visit fewer nodes one
-// after another.  Measured on the city frame (acceptance stage): 1 piece
-// 0.22 ms, 2 0.20, 4 0.17, 8 0.17, 16 0.20; the same records.
-constexpr uint32_t kOcclPieces = 4;
+// Each leg's any-hit test is split into pieces of t in (0, 1) on the same ray
+// (so every t is the one the whole leg would compute), one thread each: the
+// leg is occluded iff some piece is.  With the candidates of a frame the launch
+// is bound by the latency of its longest chains of node visits (first legs
+// across the city), so a piece is at most kOcclMetres long, from kOcclLeast up
+// to kOcclMost pieces a leg.  With more than kOcclFull records kOcclLeast pieces
+// alone fill the GPU and further ones only add visits: the city's 40000 lines
+// of sight (emrt_refresh_schedule) take 193 us of update and schedule with 4
+// pieces, 259 with up to 16.  A block takes kOcclLegs legs (leg-major: the
+// first legs, the longest, first), counts their pieces and hands them to its
+// threads, so legs that are not there (shallower or rejected paths) take no
+// thread.  City frame, acceptance of 16k candidates (geometry included): 152
+// us with 4 pieces and a thread for every possible leg, 134 with the legs
+// packed and the FP32 margin above, 113 with pieces of 64 m (32 m: 115);
+// district 68 -> 59.  The compressed 8-wide tree (128 on the city) and a thread
+// each for triangles and vehicles (111; district 64 against 59) are not used.
+constexpr uint32_t kOcclLegs = 32, kOcclLeast = 4, kOcclMost = 16, kOcclFull = 32768;
+constexpr float kOcclMetres = 64.f;
+static_assert(kOcclLegs == 32, "a block's legs are counted by its first warp");
 template <bool BATCH>
 __global__ void __launch_bounds__(kBounceBlock) k_accept_occl(GeomView G, const BatchScene *__restrict__ tab,
                                                               uint32_t *rec, const uint32_t *n,
                                                               const float4 *pts, uint32_t cap,
                                                               Counters *ctr) {
+  __shared__ uint32_t s_first[kOcclLegs + 1];  // pieces before a leg of the block
   StackSlot stk[kStack];
   TravStats st;
   const uint32_t cnt = min(*n, cap);
   const uint32_t NO = EMRT_NO_FACE;
   unsigned long long occl = 0;
-  const uint64_t items = (uint64_t)(EMRT_MAX_DEPTH + 1) * cnt * kOcclPieces;
-  for (uint64_t it = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; it < items;
-       it += (uint64_t)gridDim.x * blockDim.x) {
-    const uint32_t piece = (uint32_t)(it % kOcclPieces);
-    const uint64_t leg = it / kOcclPieces;
-    const uint32_t q = (uint32_t)(leg / cnt), i = (uint32_t)(leg - (uint64_t)q * cnt);
-    const uint4 *r = reinterpret_cast<const uint4 *>(rec + 8ull * i);
-    const uint4 a = r[0];
-    const uint32_t k = a.z & 15u;
-    if (q > k || !(a.z & EMRT_PATH_VALID)) continue;
-    const uint4 b = r[1];
-    const uint32_t f[EMRT_MAX_DEPTH] = {a.w, b.x, b.y, b.z};
-    const uint32_t sc = BATCH ? (a.x >> 8) : 0u;
-    const GeomView &g = BATCH ? tab[sc].g : G;
-    const float3 A = f3(pts[(uint64_t)q * cap + i]), B = f3(pts[(uint64_t)(q + 1) * cap + i]);
-    const uint32_t e0 = q >= 1 ? f[q - 1] : NO, e1 = q < k ? f[q] : NO;
-    const uint32_t v0 = (e0 != NO && e0 >= g.n_static_faces) ? (e0 - g.n_static_faces) / 6u : NO;
-    const uint32_t v1 = (e1 != NO && e1 >= g.n_static_faces) ? (e1 - g.n_static_faces) / 6u : NO;
-    RayQ rq;
-    ray_setup(rq, A, B - A);
-    // this piece's share of t in (0, 1); neighbouring pieces overlap by a
-    // relative 2^-20 so that a hit exactly at a boundary falls in one of them
-    const float hi = piece + 1u == kOcclPieces ? 1.f : (float)(piece + 1u) / kOcclPieces;
-    const float lo = piece == 0u ? 0.f : (float)piece / kOcclPieces * (1.f - 9.5367431640625e-7f);
-    float tmax = hi;
-    uint32_t hf = NO;
-    occl++;
-    bool hit = trace_tris<true>(g.stat, rq, lo, tmax, hf, e0, e1, stk, st);
-    tmax = hi;
-    if (!hit) hit = trace_boxes<true>(g.dyn, rq, lo, tmax, hf, g.n_static_faces, v0, v1, stk, st);
-    if (hit) atomicAnd(&rec[8ull * i + 2], ~EMRT_PATH_VALID);
+  const uint64_t legs = (uint64_t)(EMRT_MAX_DEPTH + 1) * cnt;
+  for (uint64_t base = (uint64_t)blockIdx.x * kOcclLegs; base < legs;
+       base += (uint64_t)gridDim.x * kOcclLegs) {
+    if (threadIdx.x < kOcclLegs) {
+      uint32_t pieces = 0;
+      const uint64_t leg = base + threadIdx.x;
+      if (leg < legs) {
+        const uint32_t q = (uint32_t)(leg / cnt), i = (uint32_t)(leg - (uint64_t)q * cnt);
+        const uint32_t w2 = rec[8ull * i + 2];
+        if (q <= (w2 & 15u) && (w2 & EMRT_PATH_VALID)) {
+          const float3 d = f3(pts[(uint64_t)(q + 1) * cap + i]) - f3(pts[(uint64_t)q * cap + i]);
+          const float len = sqrtf(dot3(d, d));
+          pieces = kOcclLeast;
+          if (cnt <= kOcclFull)
+            pieces = (uint32_t)fminf(fmaxf(ceilf(len * (1.f / kOcclMetres)), (float)kOcclLeast),
+                                     (float)kOcclMost);
+        }
+      }
+      uint32_t incl = pieces;
+      const uint32_t lane = threadIdx.x & 31;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
+      }
+      s_first[threadIdx.x + 1] = incl;
+      if (threadIdx.x == 0) s_first[0] = 0;
+    }
+    __syncthreads();
+    const uint32_t total = s_first[kOcclLegs];
+    for (uint32_t w = threadIdx.x; w < total; w += kBounceBlock) {
+      uint32_t lo_leg = 0, hi_leg = kOcclLegs;  // last leg starting at or before piece w
+      while (hi_leg - lo_leg > 1) {
+        const uint32_t mid = (lo_leg + hi_leg) >> 1;
+        if (s_first[mid] <= w) lo_leg = mid;
+        else hi_leg = mid;
+      }
+      const uint32_t pieces = s_first[lo_leg + 1] - s_first[lo_leg], piece = w - s_first[lo_leg];
+      const uint64_t leg = base + lo_leg;
+      const uint32_t q = (uint32_t)(leg / cnt), i = (uint32_t)(leg - (uint64_t)q * cnt);
+      const uint4 *r = reinterpret_cast<const uint4 *>(rec + 8ull * i);
+      const uint4 a = r[0];
+      const uint32_t k = a.z & 15u;
+      if (!(a.z & EMRT_PATH_VALID)) continue;  // another piece or leg was occluded
+      const uint4 b = r[1];
+      const uint32_t f[EMRT_MAX_DEPTH] = {a.w, b.x, b.y, b.z};
+      const uint32_t sc = BATCH ? (a.x >> 8) : 0u;
+      const GeomView &g = BATCH ? tab[sc].g : G;
+      const float3 A = f3(pts[(uint64_t)q * cap + i]), B = f3(pts[(uint64_t)(q + 1) * cap + i]);
+      const uint32_t e0 = q >= 1 ? f[q - 1] : NO, e1 = q < k ? f[q] : NO;
+      const uint32_t v0 = (e0 != NO && e0 >= g.n_static_faces) ? (e0 - g.n_static_faces) / 6u : NO;
+      const uint32_t v1 = (e1 != NO && e1 >= g.n_static_faces) ? (e1 - g.n_static_faces) / 6u : NO;
+      RayQ rq;
+      ray_setup(rq, A, B - A);
+      // this piece's share of t in (0, 1); neighbouring pieces overlap by a
+      // relative 2^-20 so that a hit exactly at a boundary falls in one of them
+      const float hi = piece + 1u == pieces ? 1.f : (float)(piece + 1u) / (float)pieces;
+      const float lo = piece == 0u ? 0.f : (float)piece / (float)pieces * (1.f - 9.5367431640625e-7f);
+      float tmax = hi;
+      uint32_t hf = NO;
+      occl++;
+      bool hit = trace_tris<true>(g.stat, rq, lo, tmax, hf, e0, e1, stk, st);
+      tmax = hi;
+      if (!hit) hit = trace_boxes<true>(g.dyn, rq, lo, tmax, hf, g.n_static_faces, v0, v1, stk, st);
+      if (hit) atomicAnd(&rec[8ull * i + 2], ~EMRT_PATH_VALID);
+    }
+    __syncthreads();
   }
   add_u64(&ctr->occl_rays, occl);
   if (st.overflow) atomicOr(&ctr->err, ERR_STACK);
