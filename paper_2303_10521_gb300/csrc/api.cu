@@ -48,7 +48,7 @@ cudaError_t grow(T **p, uint64_t &cap, uint64_t need) {
 }
 
 __global__ void k_faces(const uint32_t *off, const float *xyz, const uint32_t *mat, uint32_t F,
-                        double4_32a *plane, uint4 *info, float4 *vert) {
+                        double4_32a *plane, float4 *nf, uint4 *info, float4 *vert) {
   uint32_t f = blockIdx.x * blockDim.x + threadIdx.x;
   if (f >= F) return;
   uint32_t a = off[f], nv = off[f + 1] - off[f];
@@ -67,6 +67,7 @@ __global__ void k_faces(const uint32_t *off, const float *xyz, const uint32_t *m
   double l = sqrt(nx * nx + ny * ny + nz * nz);
   nx /= l; ny /= l; nz /= l;
   plane[f] = make_double4_32a(nx, ny, nz, (nx * cx + ny * cy + nz * cz) / nv);
+  nf[f] = make_float4((float)nx, (float)ny, (float)nz, 0.f);
   info[f] = make_uint4(a, nv, mat[f], 0u);
 }
 
@@ -216,11 +217,12 @@ emrt_status emrt_scene_create(const emrt_scene_desc *d, emrt_stream stream, emrt
     if (e) return fail(e);
   }
   if ((e = grow(&s->face_plane, c, std::max(s->Fs, 1u)))) return fail(e); c = 0;
+  if ((e = grow(&s->face_nf, c, std::max(s->Fs, 1u)))) return fail(e); c = 0;
   if ((e = grow(&s->face_info, c, std::max(s->Fs, 1u)))) return fail(e); c = 0;
   if ((e = grow(&s->face_vert, c, std::max(s->NV, 1u)))) return fail(e); c = 0;
   if ((e = grow(&s->bbox, c, 4))) return fail(e); c = 0;
   if (s->Fs) emrt::note_launch(), k_faces<<<ceil_div(s->Fs, 128), 128, 0, st>>>(d->face_off, d->face_xyz, d->face_mat,
-                                                          s->Fs, s->face_plane, s->face_info,
+                                                          s->Fs, s->face_plane, s->face_nf, s->face_info,
                                                           s->face_vert);
   if ((e = grow(&s->ctr, c, 1))) return fail(e); c = 0;
   if ((e = grow(&s->hist, c, 256 * kPrimGrid + 1))) return fail(e); c = 0;
@@ -292,7 +294,7 @@ emrt_status emrt_scene_create(const emrt_scene_desc *d, emrt_stream stream, emrt
 void emrt_scene_destroy(emrt_scene s) {
   if (!s) return;
   batch_forget_scene(s);
-  cudaFree(s->face_plane); cudaFree(s->face_info); cudaFree(s->face_vert); cudaFree(s->bbox);
+  cudaFree(s->face_plane); cudaFree(s->face_nf); cudaFree(s->face_info); cudaFree(s->face_vert); cudaFree(s->bbox);
   bvh_free(s->stat); bvh_free(s->dyn); bvh_free(s->rxb); bvh_free(s->txb); bvh_free(s->mix);
   cudaFree(s->mix_lo); cudaFree(s->mix_hi);
   frame_trees_free(s->frame_trees);
@@ -588,6 +590,7 @@ emrt_status run_trace(emrt_scene_s *s, const emrt_trace_params *p, uint64_t coun
     L.kappa = kappa;
     L.K = (int)p->max_depth;
     L.jbits = jbits;
+    L.ends_last = walk_ends_last(nrays, gt.n_rx, kappa);
     cudaEventRecord(s->evb[0], st);
     launch_walk(L, st, (p->flags & EMRT_TRACE_WIDE_BVH) != 0);
     cudaEventRecord(s->evb[1], st);
@@ -964,20 +967,21 @@ emrt_status emrt_sync(emrt_scene s, emrt_stream stream, emrt_stats *out) {
       (uint64_t)h.n_cand + h.n_cand / 4 + 1024, 0x7fffffffull);
   if (out) {
     memset(out, 0, sizeof(*out));
-    for (int b = 0; b <= EMRT_MAX_DEPTH; b++) out->segments[b] = h.segments[b];
+    const WalkStats w = walk_stats(h);
+    for (int b = 0; b <= EMRT_MAX_DEPTH; b++) out->segments[b] = w.segments[b];
     out->candidates = h.n_cand;
     out->unique_candidates = h.n_unique;
     out->accepted = h.n_accepted;
     out->occlusion_rays = h.occl_rays;
-    out->node_visits = h.node_visits;
-    out->tri_tests = h.tri_tests;
+    out->node_visits = w.node_visits;
+    out->tri_tests = w.tri_tests;
     out->error_bits = h.err;
-    out->dyn_node_visits = h.dyn_node_visits;
-    out->box_tests = h.box_tests;
-    out->rx_node_visits = h.rx_node_visits;
-    out->rx_tests = h.rx_tests;
-    out->static_reused = h.static_reused;
-    out->deferred = h.deferred;
+    out->dyn_node_visits = w.dyn_node_visits;
+    out->box_tests = w.box_tests;
+    out->rx_node_visits = w.rx_node_visits;
+    out->rx_tests = w.rx_tests;
+    out->static_reused = w.static_reused;
+    out->deferred = w.deferred;
     if (s->ev_recorded) {
       cudaEventElapsedTime(&out->traverse_ms, s->ev[0], s->ev[1]);
       cudaEventElapsedTime(&out->dedup_ms, s->ev[1], s->ev[2]);

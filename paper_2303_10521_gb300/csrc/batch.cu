@@ -130,6 +130,7 @@ void fill_table(emrt_batch_s *b) {
     t.out_rec = b->outs[i].rec;
     t.out_cap = b->outs[i].capacity;
     t.out_count = b->outs[i].count;
+    t.ends_last = walk_ends_last(b->total, t.g.n_rx, t.kappa);
     t.pair_begin = pairs;
     t.pair_rx = s->max_rx;
     pairs += b->n_tx[i] * s->max_rx;
@@ -520,17 +521,18 @@ emrt_status emrt_batch_sync(emrt_batch b, emrt_stream stream, emrt_stats *out) {
     b->want_cand = (uint32_t)std::min<uint64_t>((uint64_t)h.n_cand + h.n_cand / 4 + 1024, 0x7fffffffull);
   if (out) {
     memset(out, 0, sizeof(*out));
-    for (int k = 0; k <= EMRT_MAX_DEPTH; k++) out->segments[k] = h.segments[k];
+    const WalkStats w = walk_stats(h);
+    for (int k = 0; k <= EMRT_MAX_DEPTH; k++) out->segments[k] = w.segments[k];
     out->candidates = h.n_cand;
     out->unique_candidates = h.n_unique;
     out->accepted = h.n_accepted;
     out->occlusion_rays = h.occl_rays;
-    out->node_visits = h.node_visits;
-    out->tri_tests = h.tri_tests;
-    out->dyn_node_visits = h.dyn_node_visits;
-    out->box_tests = h.box_tests;
-    out->rx_node_visits = h.rx_node_visits;
-    out->rx_tests = h.rx_tests;
+    out->node_visits = w.node_visits;
+    out->tri_tests = w.tri_tests;
+    out->dyn_node_visits = w.dyn_node_visits;
+    out->box_tests = w.box_tests;
+    out->rx_node_visits = w.rx_node_visits;
+    out->rx_tests = w.rx_tests;
     out->error_bits = h.err;
     out->required_candidates = h.n_cand;
     out->required_paths = h.n_accepted;

@@ -4,10 +4,7 @@
 #pragma once
 
 __device__ inline float3 face_normal_f(const GeomView &g, uint32_t f) {
-  if (f < g.n_static_faces) {
-    double4_32a p = g.face_plane[f];
-    return make_float3((float)p.x, (float)p.y, (float)p.z);
-  }
+  if (f < g.n_static_faces) return f3(ldg4(g.face_nf + f));
   uint32_t j = (f - g.n_static_faces) % 6u;
   float s = (j & 1u) ? 1.f : -1.f;
   int ax = j >> 1;
@@ -29,6 +26,13 @@ __device__ inline void rx_bounds(const BVHView &b, float3 &lo, float3 &hi) {
 __device__ inline void add_u64(unsigned long long *p, unsigned long long v) {
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0 && v) atomicAdd(p, v);
+}
+
+// The copy of ctr's statistics that this warp adds to at the end of a traversal
+// kernel, one add_u64() a counter.
+__device__ inline WalkStats *walk_copy(Counters *ctr) {
+  const uint32_t warp = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+  return ctr->walk + warp % kStatCopies;
 }
 
 // Specular continuation of a segment that hit `face` at t: hit point p and
@@ -208,12 +212,13 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_bounce(BounceLaunch L, 
     }
   }
   __syncwarp();
-  add_u64(&L.ctr->segments[L.b], segs);
-  add_u64(&L.ctr->node_visits, st.nodes);
-  add_u64(&L.ctr->tri_tests, st.tris);
-  add_u64(&L.ctr->dyn_node_visits, st.dnodes);
-  add_u64(&L.ctr->box_tests, st.boxes);
-  add_u64(&L.ctr->rx_node_visits, st.rnodes);
-  add_u64(&L.ctr->rx_tests, st.rxs);
+  WalkStats *w = walk_copy(L.ctr);
+  add_u64(&w->segments[L.b], segs);
+  add_u64(&w->node_visits, st.nodes);
+  add_u64(&w->tri_tests, st.tris);
+  add_u64(&w->dyn_node_visits, st.dnodes);
+  add_u64(&w->box_tests, st.boxes);
+  add_u64(&w->rx_node_visits, st.rnodes);
+  add_u64(&w->rx_tests, st.rxs);
   if (st.overflow) atomicOr(&L.ctr->err, ERR_STACK);
 }

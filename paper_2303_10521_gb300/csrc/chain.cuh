@@ -4,6 +4,29 @@
 // its anonymous namespace.
 #pragma once
 
+// Items of a persistent launch, 32 neighbours at a time: a warp's first 32 are
+// its own by position, the next come from the cursor.  A launch with no more
+// items than threads takes no atomic (6080 warps asking one address for work
+// cost it about 6 us).
+struct WorkItems {
+  uint32_t base;  // warp-uniform
+  bool first = true;
+  __device__ bool next(uint32_t *cursor, uint32_t n) {
+    const uint32_t threads = gridDim.x * blockDim.x;
+    if (first) {
+      first = false;
+      base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
+      return base < n;
+    }
+    if (threads >= n) return false;
+    uint32_t b = 0;
+    if ((threadIdx.x & 31) == 0) b = atomicAdd(cursor, 32u);
+    b = __shfl_sync(0xffffffffu, b, 0);
+    base = b + threads;
+    return b < n - threads;
+  }
+};
+
 // One chain from its first unfinished segment to its end, in scene g (kappa:
 // reception radius factor, K: reflections).  CACHE (single scene): static
 // hit from the cache L.stab while the chain is still static and its entry
@@ -16,7 +39,7 @@
 // Segments, candidates and cache entries are exactly those of k_bounce.
 template <bool CACHE, bool WIDE = false>
 __device__ __forceinline__ void carry_chain(const BounceLaunch &L, const GeomView &g, float kappa,
-                                            int K, uint32_t w0, uint32_t tx, uint32_t item,
+                                            int K, bool ends_last, uint32_t w0, uint32_t tx, uint32_t item,
                                             uint32_t jj, const Ray &R, float3 rlo, float3 rhi,
                                             StackSlot *stk, TravStats &st,
                                             uint32_t (&segs)[EMRT_MAX_DEPTH + 1],
@@ -47,6 +70,15 @@ __device__ __forceinline__ void carry_chain(const BounceLaunch &L, const GeomVie
         have = true;
         reused++;
       }
+    }
+    // the last segment of a chain only matters where it is received: where no
+    // receiver can be, its end need not be known
+    if (!CACHE && ends_last && (int)b >= K &&
+        !rx_possible(g.rxb, q, fmaxf(escape_t(o, d, rlo, rhi), 0.f), Lacc, kappa, stk, st)) {
+#pragma unroll
+      for (uint32_t k = 0; k <= EMRT_MAX_DEPTH; k++)
+        if (k == b) segs[k]++;
+      break;
     }
     if (!have) {
       trace_tris<false, WIDE>(g.stat, q, 0.f, tbest, face, prev, NO, stk, st);
@@ -88,7 +120,7 @@ __device__ __forceinline__ void carry_queued(const BounceLaunch &L, const Ray &R
                                              uint32_t &reused) {
   const uint32_t id = __float_as_uint(R.d_id.w);
   const uint32_t tx = id >> L.jbits, pos = id & ((1u << L.jbits) - 1u);
-  carry_chain<true>(L, L.g, L.kappa, L.K, tx, tx, tx * L.count + pos,
+  carry_chain<true>(L, L.g, L.kappa, L.K, false, tx, tx, tx * L.count + pos,
                     __float_as_uint(L.dirs[pos].w), R, rlo, rhi, stk, st, segs, reused);
 }
 
@@ -102,9 +134,11 @@ __device__ __forceinline__ void carry_queued(const BounceLaunch &L, const Ray &R
 // as it holds 32 chains the warp carries them to their ends together
 // (carry_chain), so that the costly deferred segments run while the walk
 // still fills the GPU, 32 to a warp, rather than in a sparse launch of their
-// own.  The queue's last chains are carried when the walk is handed out.
+// own.  The queue's last chains are carried when the walk is handed out.  56
+// registers (9 blocks of 128 an SM): city 2.22 ms, at N/10 0.51 (48: 2.27 and
+// 0.52; 64: 2.20 and 0.53).
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_chain(BounceLaunch L, ChainBufs D) {
+__global__ void __launch_bounds__(BLOCK, 1152 / BLOCK) k_chain(BounceLaunch L, ChainBufs D) {
   StackSlot stk[kStack];
   TravStats st;
   uint32_t segs[EMRT_MAX_DEPTH + 1] = {0, 0, 0, 0, 0};
@@ -117,12 +151,8 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_chain(BounceLaunch L, C
   uint32_t qn = 0;  // chains in the warp's queue (warp-uniform)
   float3 rlo, rhi;
   rx_bounds(L.g.rxb, rlo, rhi);
-  for (;;) {
-    uint32_t base = 0;
-    if (lane == 0) base = atomicAdd(L.work, 32u);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (base >= n_items) break;
-    const uint32_t i = base + lane;
+  for (WorkItems work; work.next(L.work, n_items);) {
+    const uint32_t i = work.base + lane;
     bool defer = false;
     float3 o, d;
     float Lacc = 0.f;
@@ -195,15 +225,16 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_chain(BounceLaunch L, C
   __syncwarp();
   if (lane < qn) carry_queued(L, wq[lane], rlo, rhi, stk, st, segs, reused);
   __syncwarp();
-  for (int b = 0; b <= EMRT_MAX_DEPTH; b++) add_u64(&L.ctr->segments[b], segs[b]);
-  add_u64(&L.ctr->node_visits, st.nodes);
-  add_u64(&L.ctr->tri_tests, st.tris);
-  add_u64(&L.ctr->dyn_node_visits, st.dnodes);
-  add_u64(&L.ctr->box_tests, st.boxes);
-  add_u64(&L.ctr->rx_node_visits, st.rnodes);
-  add_u64(&L.ctr->rx_tests, st.rxs);
-  add_u64(&L.ctr->static_reused, reused);
-  add_u64(&L.ctr->deferred, deferred);
+  WalkStats *w = walk_copy(L.ctr);
+  for (int k = 0; k <= EMRT_MAX_DEPTH; k++) add_u64(&w->segments[k], segs[k]);
+  add_u64(&w->node_visits, st.nodes);
+  add_u64(&w->tri_tests, st.tris);
+  add_u64(&w->dyn_node_visits, st.dnodes);
+  add_u64(&w->box_tests, st.boxes);
+  add_u64(&w->rx_node_visits, st.rnodes);
+  add_u64(&w->rx_tests, st.rxs);
+  add_u64(&w->static_reused, reused);
+  add_u64(&w->deferred, deferred);
   if (st.overflow) atomicOr(&L.ctr->err, ERR_STACK);
 }
 
@@ -218,10 +249,13 @@ __global__ void __launch_bounds__(BLOCK, 1280 / BLOCK) k_chain(BounceLaunch L, C
 // a warp.  BATCH: primary items of many scenes (table tab, each item's scene
 // the last whose range starts at or before it; candidates carry
 // scene << 8 | tx); otherwise the single scene in L.g.  Segments and
-// candidates are exactly those of k_bounce.  WIDE: closest hits through the
+// candidates are exactly those of k_bounce.  Registers: 48 (10 blocks of 128 an
+// SM) for one scene (city 7.80 ms; 56: 8.01, 64: 8.17); 56 for a batch, whose
+// scene table takes more (12 uneven scenes 4.26 ms with the tail; 64: 4.37; at
+// 48 the compiler kept what the node loop reads in memory: 18.8).  WIDE: closest hits through the
 // compressed 8-wide tree of the static geometry (same hits).
 template <int BLOCK, bool BATCH, bool WIDE = false>
-__global__ void __launch_bounds__(BLOCK, (WIDE ? 1024 : 1280) / BLOCK) k_walk(BounceLaunch L,
+__global__ void __launch_bounds__(BLOCK, (WIDE ? 1024 : BATCH ? 1152 : 1280) / BLOCK) k_walk(BounceLaunch L,
                                                              const BatchScene *__restrict__ tab,
                                                              uint32_t n_scenes) {
   StackSlot stk[kStack];
@@ -233,12 +267,8 @@ __global__ void __launch_bounds__(BLOCK, (WIDE ? 1024 : 1280) / BLOCK) k_walk(Bo
   const uint32_t NO = EMRT_NO_FACE;
   float3 rlo, rhi;
   if (!BATCH) rx_bounds(L.g.rxb, rlo, rhi);
-  for (;;) {
-    uint32_t base = 0;
-    if (lane == 0) base = atomicAdd(L.work, 32u);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (base >= n_items) break;
-    const uint32_t i = base + lane;
+  for (WorkItems work; work.next(L.work, n_items);) {
+    const uint32_t i = work.base + lane;
     if (i < n_items) {
       uint32_t sc = 0, local = i, count = L.count;
       const float4 *dirs = L.dirs;
@@ -264,18 +294,20 @@ __global__ void __launch_bounds__(BLOCK, (WIDE ? 1024 : 1280) / BLOCK) k_walk(Bo
       R.d_id = dj;
       R.faces = make_uint4(NO, NO, NO, NO);
       carry_chain<false, WIDE>(L, g, BATCH ? tab[sc].kappa : L.kappa, BATCH ? (int)tab[sc].K : L.K,
+                         BATCH ? tab[sc].ends_last != 0 : L.ends_last != 0,
                          BATCH ? (sc << 8 | tx) : tx, tx, local, __float_as_uint(dj.w), R, rlo,
                          rhi, stk, st, segs, unused);
     }
     __syncwarp();
   }
-  for (int k = 0; k <= EMRT_MAX_DEPTH; k++) add_u64(&L.ctr->segments[k], segs[k]);
-  add_u64(&L.ctr->node_visits, st.nodes);
-  add_u64(&L.ctr->tri_tests, st.tris);
-  add_u64(&L.ctr->dyn_node_visits, st.dnodes);
-  add_u64(&L.ctr->box_tests, st.boxes);
-  add_u64(&L.ctr->rx_node_visits, st.rnodes);
-  add_u64(&L.ctr->rx_tests, st.rxs);
+  WalkStats *w = walk_copy(L.ctr);
+  for (int k = 0; k <= EMRT_MAX_DEPTH; k++) add_u64(&w->segments[k], segs[k]);
+  add_u64(&w->node_visits, st.nodes);
+  add_u64(&w->tri_tests, st.tris);
+  add_u64(&w->dyn_node_visits, st.dnodes);
+  add_u64(&w->box_tests, st.boxes);
+  add_u64(&w->rx_node_visits, st.rnodes);
+  add_u64(&w->rx_tests, st.rxs);
   if (st.overflow) atomicOr(&L.ctr->err, ERR_STACK);
 }
 

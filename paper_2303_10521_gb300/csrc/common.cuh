@@ -18,6 +18,25 @@ enum : uint32_t {
   ERR_WAIT = 64u,           // a bounded wait between blocks gave up
 };
 
+// Statistics of the traversal launches.  Every warp adds its own at its end;
+// kStatCopies copies, each on a 128-byte line, keep the warps of a short
+// launch, which end together, from queueing at one address (atomics on one
+// address complete at about one a nanosecond, and a launch has 6080 warps).
+constexpr uint32_t kStatCopies = 32;
+constexpr uint32_t kWalkStats = EMRT_MAX_DEPTH + 1 + 8;
+struct alignas(128) WalkStats {
+  unsigned long long segments[EMRT_MAX_DEPTH + 1];
+  unsigned long long node_visits;     // static BVH inner nodes visited
+  unsigned long long tri_tests;       // triangles tested
+  unsigned long long dyn_node_visits; // vehicle BVH inner nodes visited
+  unsigned long long box_tests;       // vehicle boxes tested
+  unsigned long long rx_node_visits;  // receiver BVH inner nodes visited
+  unsigned long long rx_tests;        // receivers tested against a sphere
+  unsigned long long static_reused;   // static hits taken from the cache
+  unsigned long long deferred;        // chains the cache walker queued
+};
+static_assert(sizeof(unsigned long long) * kWalkStats <= 128, "one line a copy");
+
 // per-call counters kept in device memory (one struct per scene)
 struct Counters {
   uint32_t err;                            // error bits (cleared by emrt_sync)
@@ -28,17 +47,9 @@ struct Counters {
   uint32_t n_unique;
   uint32_t n_accepted;
   uint32_t tmp;
-  uint32_t chain_work;                     // work cursor of the cache walker
-  unsigned long long segments[EMRT_MAX_DEPTH + 1];
-  unsigned long long node_visits;     // static BVH inner nodes visited
-  unsigned long long tri_tests;       // triangles tested
-  unsigned long long dyn_node_visits; // vehicle BVH inner nodes visited
-  unsigned long long box_tests;       // vehicle boxes tested
-  unsigned long long rx_node_visits;  // receiver BVH inner nodes visited
-  unsigned long long rx_tests;        // receivers tested against a sphere
+  uint32_t chain_work;                     // work cursor of k_walk, k_chain
   unsigned long long occl_rays;
-  unsigned long long static_reused;   // static hits taken from the cache
-  unsigned long long deferred;        // chains the cache walker queued
+  WalkStats walk[kStatCopies];
 };
 
 // ---------------------------------------------------------------------------
@@ -157,6 +168,8 @@ struct GeomView {
   BVHView mix;             // vehicles and receivers in one tree (or empty):
                            // prims 0..n_veh-1 boxes, then receiver points
   const double4_32a *face_plane;  // [F_s] unit normal, offset
+  const float4 *face_nf;      // [F_s] the normal in FP32 (reflection: no FP64
+                              // conversion, 64 cycles each, on the chains)
   const uint4 *face_info;     // [F_s] vertex offset, vertex count, material, 0
   const float4 *face_vert;    // [NV] polygon vertices
   const float4 *veh_lo;       // [V] box corners (w unused)
@@ -170,6 +183,17 @@ struct GeomView {
 };
 
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
+
+// the copies' sum (host side)
+inline WalkStats walk_stats(const Counters &c) {
+  WalkStats w{};
+  unsigned long long *o = w.segments;
+  for (uint32_t k = 0; k < kStatCopies; k++) {
+    const unsigned long long *v = c.walk[k].segments;
+    for (uint32_t q = 0; q < kWalkStats; q++) o[q] += v[q];
+  }
+  return w;
+}
 
 // host-side count of kernel launches issued by this library (diagnostics)
 void note_launch();

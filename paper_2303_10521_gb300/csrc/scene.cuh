@@ -12,7 +12,7 @@ struct emrt_scene_s {
   uint32_t rebuild_every = 1, n_updates = 0;
   double4_32a *face_plane = nullptr;
   uint4 *face_info = nullptr;
-  float4 *face_vert = nullptr;
+  float4 *face_vert = nullptr, *face_nf = nullptr;
   float4 *bbox = nullptr;  // [4]: lo, hi, scratch
   BVHBuf stat, dyn, rxb;
   BVHBuf txb;                     // transmitter points (backward tracing)
@@ -94,6 +94,7 @@ inline GeomView geom(const emrt_scene_s *s) {
   g.rxb = s->rxb.view();
   g.mix = s->mix.view();
   g.face_plane = s->face_plane;
+  g.face_nf = s->face_nf;
   g.face_info = s->face_info;
   g.face_vert = s->face_vert;
   g.veh_lo = s->veh_lo;

@@ -1,7 +1,7 @@
 // Discovery (shoot-and-bounce with reception spheres) and image-method
 // acceptance kernels.
+#include <algorithm>
 #include <cfloat>
-
 #include <cstring>
 
 #include "trace.cuh"
@@ -575,7 +575,8 @@ uint64_t chain_queue_entries() {
 }
 
 void launch_chain(const BounceLaunch &L, const ChainBufs &D, int grid, cudaStream_t s) {
-  emrt::note_launch(), k_chain<kBounceBlock><<<grid, kBounceBlock, 0, s>>>(L, D);
+  const int blocks = std::min(grid, ceil_div(L.n_primary, kBounceBlock));
+  emrt::note_launch(), k_chain<kBounceBlock><<<blocks, kBounceBlock, 0, s>>>(L, D);
 }
 
 int g_walk_grid[2] = {0, 0};
@@ -592,11 +593,25 @@ int walk_grid() {
   return g_walk_grid[WIDE];
 }
 
+// The query costs a traversal of the receiver tree over the whole ray and saves
+// the static and merged traversals of the segments that no receiver is near.
+// n_rx kappa is the expected number of receivers whose sphere a ray across the
+// scene meets.  Walk with the query against without (city of 10-40 blocks, 1e2-
+// 1e4 receivers, K = 4 / K = 2): n_rx kappa up to 2 1.04-1.13x / 1.05-1.30x at
+// any ray count (0.4M-32M), 3.9 0.97-1.03x / 1.04-1.13x, 8.7 at 0.4M rays (one
+// round of warps, bound by its longest chains) 0.84-0.89x, 9.7 at 32M rays
+// 1.03-1.04x / 1.13x, 19 0.94-1.00x, 39 0.77-0.87x.
+bool walk_ends_last(uint64_t n_rays_launched, uint32_t n_rx, float kappa) {
+  const float met = (float)n_rx * kappa;
+  return met <= 2.5f || (met <= 10.f && n_rays_launched >= (1u << 24));
+}
+
 void launch_walk(const BounceLaunch &L, cudaStream_t s, bool wide) {
+  const int need = ceil_div(L.n_primary, kBounceBlock);
   if (wide)
-    emrt::note_launch(), k_walk<kBounceBlock, false, true><<<walk_grid<true>(), kBounceBlock, 0, s>>>(L, nullptr, 1);
+    emrt::note_launch(), k_walk<kBounceBlock, false, true><<<std::min(need, walk_grid<true>()), kBounceBlock, 0, s>>>(L, nullptr, 1);
   else
-    emrt::note_launch(), k_walk<kBounceBlock, false><<<walk_grid<false>(), kBounceBlock, 0, s>>>(L, nullptr, 1);
+    emrt::note_launch(), k_walk<kBounceBlock, false><<<std::min(need, walk_grid<false>()), kBounceBlock, 0, s>>>(L, nullptr, 1);
 }
 
 void launch_tx_epoch(const float4 *pos, float4 *ref, uint32_t *epoch, uint32_t n_tx,

@@ -35,6 +35,7 @@ struct BounceLaunch {
   Counters *ctr;
   float kappa;
   int b, K;
+  int ends_last;         // k_walk: see walk_ends_last
   int jbits;             // single-scene ray ids: source << jbits | ray index j
   // static-hit cache (chain walker): entry (bounce b, item i) at
   // stab[b * n_slots + i], item i = tx * count + position in the direction
@@ -56,6 +57,9 @@ constexpr uint32_t kChainQueue = 64;
 struct ChainBufs {
   Ray *q;
 };
+// Whether k_walk asks for possible receivers before it looks for the end of a
+// chain's last segment.
+bool walk_ends_last(uint64_t n_rays_launched, uint32_t n_rx, float kappa);
 uint64_t chain_queue_entries();
 void launch_chain(const BounceLaunch &L, const ChainBufs &D, int grid, cudaStream_t s);
 int chain_grid();
@@ -86,6 +90,7 @@ struct BatchScene {
   uint32_t *out_rec;      // caller's output records
   uint32_t out_cap;
   uint32_t *out_count;
+  int ends_last;          // see walk_ends_last
   uint32_t pair_begin;    // first pair of this scene in the batch's pair space
   uint32_t pair_rx;       // its receiver capacity (pairs of a transmitter)
 };

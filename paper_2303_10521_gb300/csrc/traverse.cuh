@@ -9,6 +9,8 @@
 // FMA contraction (so both triangles sharing an edge see the same value) and
 // re-evaluate them in double precision when one of them is exactly zero.
 #pragma once
+#include <cfloat>
+
 #include "common.cuh"
 
 namespace emrt {
@@ -529,6 +531,63 @@ __device__ inline void trace_veh_rx(const BVHView &b, const RayQ &r, float &tmax
     }
     node = stk[sp].node;
     tcur = stk[sp].t;
+  }
+}
+
+// Whether some receiver may be detected on the segment that starts at r.o, L
+// travelled, wherever it ends: a conservative form of rx_hit() without the
+// segment's end.  A receiver detected on [0, t_end] lies within kappa (L + s)
+// of the ray at its own projection s: when the projection lies beyond t_end, its
+// distance from the ray is no larger than from the segment's end and the radius
+// has grown.  The boxes are grown by the radius at tmax, a bound of every
+// receiver's projection, and all radii by 2^-8, far above the rounding of
+// either form.
+__device__ inline bool rx_possible(const BVHView &b, const RayQ &r, float tmax, float L, float kappa,
+                                   StackSlot *stk, TravStats &st) {
+  if (b.n_prims == 0) return false;
+  const float grown = kappa * 1.00390625f, rmax = grown * (L + tmax) + 1e-5f;
+  const float3 ol = make_float3(r.ood.x + rmax * r.idir.x, r.ood.y + rmax * r.idir.y,
+                                r.ood.z + rmax * r.idir.z);
+  const float3 oh = make_float3(r.ood.x - rmax * r.idir.x, r.ood.y - rmax * r.idir.y,
+                                r.ood.z - rmax * r.idir.z);
+  const RayPairs rp = ray_pairs_lh(r.idir, ol, oh);
+  int sp = 0;
+  int node = b.root;
+  uint32_t iter = 0;
+  for (;;) {
+    if (++iter > kMaxIter) {
+      st.overflow = true;
+      return true;
+    }
+    if (node >= 0) {
+      const float4 *np = b.nodes + 4ll * node;
+      float4 n0 = ldg4(np), n1 = ldg4(np + 1), n2 = ldg4(np + 2), n3 = ldg4(np + 3);
+      st.rnodes++;
+      float tn0, tn1;
+      const bool h0 = slab_p(rp, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, 0.f, FLT_MAX, tn0);
+      const bool h1 = slab_p(rp, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, 0.f, FLT_MAX, tn1);
+      const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
+      if (h0 && h1) {
+        if (sp >= kStack) return true;
+        stk[sp++].node = c1;
+        node = c0;
+        continue;
+      }
+      if (h0 || h1) {
+        node = h0 ? c0 : c1;
+        continue;
+      }
+    } else {
+      const float4 p = ldg4(b.prims + (uint32_t)(~node));
+      st.rxs++;
+      const float3 w = f3(p) - r.o;
+      const float s = fmaxf(dot3(w, r.d), 0.f);
+      const float3 q = w - r.d * s;
+      const float rad = grown * (L + s) + 1e-5f;
+      if (!(dot3(q, q) > rad * rad)) return true;
+    }
+    if (sp == 0) return false;
+    node = stk[--sp].node;
   }
 }
 
