@@ -141,7 +141,7 @@ void emrt_scene_destroy(emrt_scene sc);
  * tx_pos/tx_vel [n_tx][3].  Refits the vehicle BVH (rebuilds it every
  * rebuild_every calls) and rebuilds the receiver BVH and the merged
  * vehicle + receiver BVH.  Up to 32768 vehicles and receivers the trees are
- * built together in four launches; of a larger frame, trees of 4097-65536
+ * built together in one or four launches; of a larger frame, trees of 4097-65536
  * primitives are built in one cooperative launch whose blocks wait on one
  * another at a bounded grid barrier; a barrier that gives up makes the next
  * emrt_sync return

@@ -344,15 +344,16 @@ emrt_status emrt_scene_update_dynamic(emrt_scene s, const float *veh_pos, const 
   uint32_t m = std::max(s->V, std::max(n_rx, n_tx));
   const uint32_t nm = s->V + n_rx;
   const bool together = nm <= kFrameTreesMax;
-  if (together) CK(cudaMemsetAsync(s->frame_trees.count, 0, sizeof(uint32_t) * 2 * kTreeBins, st));
+  const bool binned = together && nm > kSmallFrame;
+  if (binned) CK(cudaMemsetAsync(s->frame_trees.count, 0, sizeof(uint32_t) * 2 * kTreeBins, st));
   emrt::note_launch(), k_update<<<ceil_div(m, 256), 256, 0, st>>>(veh_pos, veh_vel, s->veh_half, s->V, s->veh_lo,
                                              s->veh_hi, s->veh_vel, rx_pos, rx_vel, n_rx,
                                              s->rx_pos, s->rx_vel, tx_pos, tx_vel, n_tx, s->tx_pos,
-                                             s->tx_vel, s->bbox, s->frame_trees, together);
+                                             s->tx_vel, s->bbox, s->frame_trees, binned);
   const bool rebuild = s->n_updates % s->rebuild_every == 0;
   if (together) {
     CK(frame_trees_build(s->frame_trees, s->dyn, s->rxb, s->mix, s->veh_lo, s->veh_hi, s->V,
-                         rebuild, s->rx_pos, n_rx, st));
+                         rebuild, s->rx_pos, n_rx, s->bbox, st));
     if (s->V && !rebuild) CK(bvh_refit_boxes(s->dyn, s->veh_lo, s->veh_hi, st));
     s->n_updates++;
     s->updated = true;

@@ -87,14 +87,18 @@ constexpr uint32_t kTreeBins = 4096, kTreeBinShift = 18;
 // together: the codes of the widest tree have to fit a block's shared memory
 // (128 KB here); at 32760 the update takes 54 us against 126 us.
 constexpr uint32_t kFrameTreesMax = 32768;
+// ... and up to which one block a tree builds them in one launch
+constexpr uint32_t kSmallFrame = 2048;
 cudaError_t frame_trees_alloc(FrameTreesBuf &b, uint32_t n);
 void frame_trees_free(FrameTreesBuf &b);
 // Builds the receiver tree, the merged tree and, when `vehicles`, the vehicle
-// tree of a frame of V + R <= min(f.cap, kFrameTreesMax) primitives whose
-// codes, places and bin counts are at f (see frame_code in lbvh.cuh).
+// tree of a frame of V + R <= min(f.cap, kFrameTreesMax) primitives; above
+// kSmallFrame their codes, places and bin counts are at f (see frame_code in
+// lbvh.cuh).
 cudaError_t frame_trees_build(const FrameTreesBuf &f, BVHBuf &veh, BVHBuf &rx, BVHBuf &mix,
                               const float4 *veh_lo, const float4 *veh_hi, uint32_t V,
-                              bool vehicles, const float4 *rx_pos, uint32_t R, cudaStream_t s);
+                              bool vehicles, const float4 *rx_pos, uint32_t R,
+                              const float4 *bbox, cudaStream_t s);
 
 // Runs the per-frame builds' grid barrier once in a cooperative launch of 4
 // blocks expecting 4 + missing arrivals (synchronous): passed = blocks that

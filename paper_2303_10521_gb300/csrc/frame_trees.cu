@@ -1,5 +1,6 @@
 // The three per-frame trees (vehicles, receivers, both merged) of up to
-// kFrameTreesMax primitives, built together in four launches.  Same trees as
+// kFrameTreesMax primitives, built together in four launches (one up to
+// kSmallFrame: k_tree_small).  Same trees as
 // the one-block, cooperative and device-wide builders of bvh.cu: the order by
 // (Morton code, index), the radix tree over it, and boxes that are exact
 // minima and maxima.
@@ -236,24 +237,22 @@ __global__ void __launch_bounds__(kBlocksBlock) k_tree_blocks(TreeSet S) {
 // Boxes of leaves first..split and split + 1..last: the aligned blocks they
 // are made of, at most two a level each and the run of the top level.  Both
 // ranges go up the levels together and a level's loads are issued before its
-// merges: the loads' latency is the time of this step.
-__device__ inline void range_boxes(const TreeView &t, const NodeRange &r, LoHi &a, LoHi &b) {
+// merges: the loads' latency is the time of this step.  at(level, i): box of
+// block i of a level.
+template <typename At>
+__device__ inline void range_boxes(At at, int top, const NodeRange &r, LoHi &a, LoHi &b) {
   a = b = no_box();
-  uint32_t l0 = r.first, r0 = r.split + 1, l1 = r.split + 1, r1 = r.last + 1, offset = 0;
+  uint32_t l0 = r.first, r0 = r.split + 1, l1 = r.split + 1, r1 = r.last + 1;
   for (int level = 0; l0 < r0 || l1 < r1; level++) {
-    auto at = [&](bool take, uint32_t i) {
-      if (!take) return no_box();
-      if (level == 0) return leaf_of(t, i);
-      return LoHi{f3(t.blocks[2ull * (offset + i)]), f3(t.blocks[2ull * (offset + i) + 1])};
-    };
-    if (level == kLevels) {
-      for (; l0 < r0; l0++) merge(a, at(true, l0));
-      for (; l1 < r1; l1++) merge(b, at(true, l1));
+    if (level == top) {
+      for (; l0 < r0; l0++) merge(a, at(level, l0));
+      for (; l1 < r1; l1++) merge(b, at(level, l1));
       break;
     }
     const bool la = l0 < r0 && (l0 & 1u), ra = l0 + la < r0 && (r0 & 1u);
     const bool lb = l1 < r1 && (l1 & 1u), rb = l1 + lb < r1 && (r1 & 1u);
-    const LoHi x = at(la, l0), y = at(ra, r0 - 1), z = at(lb, l1), w = at(rb, r1 - 1);
+    const LoHi x = la ? at(level, l0) : no_box(), y = ra ? at(level, r0 - 1) : no_box();
+    const LoHi z = lb ? at(level, l1) : no_box(), w = rb ? at(level, r1 - 1) : no_box();
     merge(a, x);
     merge(a, y);
     merge(b, z);
@@ -262,8 +261,13 @@ __device__ inline void range_boxes(const TreeView &t, const NodeRange &r, LoHi &
     r0 >>= 1;
     l1 = (l1 + 1) >> 1;
     r1 >>= 1;
-    if (level > 0) offset += (t.n + (1u << level) - 1) >> level;
   }
+}
+
+__device__ inline void put_boxes(float4 *n, const LoHi &a, const LoHi &b, float pad) {
+  n[0] = make_float4(a.lo.x - pad, a.hi.x + pad, a.lo.y - pad, a.hi.y + pad);
+  n[1] = make_float4(b.lo.x - pad, b.hi.x + pad, b.lo.y - pad, b.hi.y + pad);
+  n[2] = make_float4(a.lo.z - pad, a.hi.z + pad, b.lo.z - pad, b.hi.z + pad);
 }
 
 // One thread an inner node: its range and split from the codes in shared
@@ -283,12 +287,138 @@ __global__ void __launch_bounds__(kNodesBlock) k_tree_nodes(TreeSet S, float pad
   if (i + 1 >= t.n) return;
   const NodeRange r = hierarchy_node([](int q) { return s_codes[q]; }, (int)t.n, (int)i,
                                      t.nodes, t.leaf_parent);
+  // the levels' offsets, in step with the level asked for (each level once)
+  uint32_t offset = 0;
+  int known = 1;
+  auto at = [&](int level, uint32_t k) {
+    if (level == 0) return leaf_of(t, k);
+    for (; known < level; known++) offset += (t.n + (1u << known) - 1) >> known;
+    return LoHi{f3(t.blocks[2ull * (offset + k)]), f3(t.blocks[2ull * (offset + k) + 1])};
+  };
   LoHi a, b;
-  range_boxes(t, r, a, b);
-  float4 *n = t.nodes + 4ull * i;
-  n[0] = make_float4(a.lo.x - pad, a.hi.x + pad, a.lo.y - pad, a.hi.y + pad);
-  n[1] = make_float4(b.lo.x - pad, b.hi.x + pad, b.lo.y - pad, b.hi.y + pad);
-  n[2] = make_float4(a.lo.z - pad, a.hi.z + pad, b.lo.z - pad, b.hi.z + pad);
+  range_boxes(at, kLevels, r, a, b);
+  put_boxes(t.nodes + 4ull * i, a, b, pad);
+}
+
+// The same steps for a frame of up to kSmallFrame primitives, a block a tree
+// with bins, lists, codes and boxes in shared memory: one launch instead of
+// four (and no counts in the update), whose latencies are the time of a small
+// frame's trees.  Update (graph / call by call): 16 primitives 22.7 -> 12.4 us /
+// 34 -> 20, 1200 28.8 -> 26.7 / 40 -> 27, 2040 30.3 -> 32.9 / 43 -> 34; one
+// block's own work is what bounds it there.
+constexpr uint32_t kSmallBlock = 1024, kSmallPer = kSmallFrame / kSmallBlock;
+constexpr uint32_t kSmallBoxes = 2 * kSmallFrame + 16;
+struct SmallShared {
+  uint32_t first[kTreeBins];
+  uint2 member[kSmallFrame];
+  uint32_t code[kSmallFrame];  // in order
+  LoHi box[kSmallBoxes];       // level 0 (leaves), 1, ...
+  uint32_t warp[32];
+};
+static_assert(kTreeBins == 4 * kSmallBlock, "four bins a thread");
+
+__global__ void __launch_bounds__(kSmallBlock) k_tree_small(FrameTreesView T, TreeSet S,
+                                                            const float4 *bb, float pad) {
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  SmallShared &s = *reinterpret_cast<SmallShared *>(s_raw);
+  TreeView t = S.t[0];
+  if (blockIdx.x == 1) t = S.t[1];
+  if (blockIdx.x == 2) t = S.t[2];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float4 *prims = blockIdx.x == 0 ? T.prims[0] : blockIdx.x == 1 ? T.prims[1] : T.prims[2];
+  if (!t.n || !prims) return;
+  // primitive e of this tree: its corners
+  auto corners = [&](uint32_t e, float4 &a, float4 &b) {
+    if (blockIdx.x == 0 || (blockIdx.x == 2 && e < T.V)) {
+      a = T.veh_lo[e];
+      b = T.veh_hi[e];
+    } else {
+      a = b = T.rx[blockIdx.x == 2 ? e - T.V : e];
+    }
+  };
+#pragma unroll
+  for (uint32_t q = 0; q < 4; q++) s.first[tid + q * kSmallBlock] = 0u;
+  __syncthreads();
+  uint32_t code[kSmallPer], slot[kSmallPer];
+#pragma unroll
+  for (uint32_t q = 0; q < kSmallPer; q++) {
+    const uint32_t e = tid + q * kSmallBlock;
+    if (e < t.n) {
+      float4 a, b;
+      corners(e, a, b);
+      code[q] = frame_code_of(a, b, bb);
+      slot[q] = atomicAdd(&s.first[code[q] >> kTreeBinShift], 1u);
+    }
+  }
+  __syncthreads();
+  {  // bins' counts to first positions, four bins a thread
+    const uint4 c = reinterpret_cast<const uint4 *>(s.first)[tid];
+    const uint32_t sum = c.x + c.y + c.z + c.w;
+    uint32_t incl = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= (uint32_t)o) incl += y;
+    }
+    if (lane == 31) s.warp[warp] = incl;
+    __syncthreads();
+    uint32_t run = incl - sum;
+    for (uint32_t w = 0; w < warp; w++) run += s.warp[w];
+    reinterpret_cast<uint4 *>(s.first)[tid] =
+        make_uint4(run, run + c.x, run + c.x + c.y, run + c.x + c.y + c.z);
+  }
+  __syncthreads();
+#pragma unroll
+  for (uint32_t q = 0; q < kSmallPer; q++) {
+    const uint32_t e = tid + q * kSmallBlock;
+    if (e < t.n) s.member[s.first[code[q] >> kTreeBinShift] + slot[q]] = make_uint2(code[q], e);
+  }
+  __syncthreads();
+  for (uint32_t i = tid; i < t.n; i += kSmallBlock) {
+    const uint2 me = s.member[i];
+    const uint32_t bin = me.x >> kTreeBinShift;
+    const uint32_t b0 = s.first[bin], b1 = bin + 1u < kTreeBins ? s.first[bin + 1u] : t.n;
+    uint32_t at = b0;
+    for (uint32_t q = b0; q < b1; q++) {
+      const uint2 m = s.member[q];
+      at += m.x < me.x || (m.x == me.x && m.y < me.y) ? 1u : 0u;  // equal codes by index
+    }
+    float4 a, b;
+    corners(me.y, a, b);
+    s.code[at] = me.x;
+    s.box[at] = LoHi{f3(a), f3(b)};
+    if (t.points) {
+      prims[at] = make_float4(a.x, a.y, a.z, __uint_as_float(me.y));
+    } else {
+      prims[2ull * at] = make_float4(a.x, a.y, a.z, __uint_as_float(me.y));
+      prims[2ull * at + 1] = make_float4(b.x, b.y, b.z, 0.f);
+    }
+  }
+  __syncthreads();
+  uint32_t below = 0, size = t.n;  // level under the one being made
+  while (size > 1u) {
+    const uint32_t up = (size + 1u) / 2u, made = below + size;
+    for (uint32_t i = tid; i < up; i += kSmallBlock) {
+      LoHi b = s.box[below + 2u * i];
+      if (2u * i + 1u < size) merge(b, s.box[below + 2u * i + 1u]);
+      s.box[made + i] = b;
+    }
+    __syncthreads();
+    below = made;
+    size = up;
+  }
+  for (uint32_t i = tid; i + 1u < t.n; i += kSmallBlock) {
+    const NodeRange r = hierarchy_node([&](int q) { return s.code[q]; }, (int)t.n, (int)i, t.nodes,
+                                       t.leaf_parent);
+    uint32_t offset = 0;
+    int known = 0;
+    auto at = [&](int level, uint32_t k) {
+      for (; known < level; known++) offset += (t.n + (1u << known) - 1u) >> known;
+      return s.box[offset + k];
+    };
+    LoHi a, b;
+    range_boxes(at, 31, r, a, b);
+    put_boxes(t.nodes + 4ull * i, a, b, pad);
+  }
 }
 
 }  // namespace
@@ -322,7 +452,8 @@ void frame_trees_free(FrameTreesBuf &b) {
 
 cudaError_t frame_trees_build(const FrameTreesBuf &f, BVHBuf &veh, BVHBuf &rx, BVHBuf &mix,
                               const float4 *veh_lo, const float4 *veh_hi, uint32_t V,
-                              bool vehicles, const float4 *rx_pos, uint32_t R, cudaStream_t s) {
+                              bool vehicles, const float4 *rx_pos, uint32_t R,
+                              const float4 *bbox, cudaStream_t s) {
   const uint32_t n = V + R;
   FrameTreesView T{};
   T.veh_lo = veh_lo;
@@ -346,6 +477,21 @@ cudaError_t frame_trees_build(const FrameTreesBuf &f, BVHBuf &veh, BVHBuf &rx, B
   if (vehicles) veh.n = V;
   rx.n = R;
   mix.n = n;
+  if (n <= kSmallFrame) {
+    TreeSet S{};
+    BVHBuf *buf[3] = {&veh, &rx, &mix};
+    for (int k = 0; k < 3; k++) {
+      S.t[k].n = k == 0 ? (vehicles ? V : 0u) : k == 1 ? R : n;
+      S.t[k].nodes = buf[k]->nodes;
+      S.t[k].leaf_parent = buf[k]->leaf_parent;
+      S.t[k].points = k == 1;
+    }
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_tree_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallShared));
+    if (e) return e;
+    emrt::note_launch(), k_tree_small<<<3, kSmallBlock, sizeof(SmallShared), s>>>(T, S, bbox, mix.pad);
+    return cudaGetLastError();
+  }
   emrt::note_launch(), k_tree_bins<<<ceil_div(n, kBinsBlock), kBinsBlock, 0, s>>>(T);
   emrt::note_launch(), k_tree_rank<<<ceil_div(n, kRankBlock), kRankBlock, 0, s>>>(T);
   TreeSet S{};

@@ -35,12 +35,15 @@ __device__ inline uint64_t morton_code(float3 p, const float4 *bb) {
 // vehicle boxes and receiver points, rebuilt every frame, use 30 (2 m cells
 // over a 2 km cube) so that their sort takes four passes instead of eight
 constexpr int kMortonBitsTri = 21, kMortonBitsDyn = 10;
-// Code of per-frame primitive i with corners a and b (a point: a = b),
-// counted in its bin (f.count zero before the first).
+// Code of a per-frame primitive with corners a and b (a point: a = b).
+__device__ inline uint32_t frame_code_of(float4 a, float4 b, const float4 *bb) {
+  return (uint32_t)morton_code<kMortonBitsDyn>(
+      make_float3(0.5f * (a.x + b.x), 0.5f * (a.y + b.y), 0.5f * (a.z + b.z)), bb);
+}
+// The code of primitive i kept and counted in its bin (f.count zero before).
 __device__ inline void frame_code(const FrameTreesBuf &f, uint32_t i, bool vehicle, float4 a,
                                   float4 b, const float4 *bb) {
-  const uint32_t code = (uint32_t)morton_code<kMortonBitsDyn>(
-      make_float3(0.5f * (a.x + b.x), 0.5f * (a.y + b.y), 0.5f * (a.z + b.z)), bb);
+  const uint32_t code = frame_code_of(a, b, bb);
   f.code[i] = code;
   f.code[f.cap + i] = atomicAdd(f.count + (code >> kTreeBinShift), 1u);
   if (vehicle) atomicAdd(f.count + kTreeBins + (code >> kTreeBinShift), 1u);

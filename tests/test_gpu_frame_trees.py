@@ -38,7 +38,8 @@ def _with_vehicles(sc, n, rng):
 
 @pytest.mark.parametrize("n_veh,n_rx,clustered", [
     (0, 1, False), (0, 2, False), (1, 1, False), (2, 3, False), (3, 512, False),
-    (511, 513, True), (512, 1024, False), (1025, 1023, True), (130, 4000, True),
+    (511, 513, True), (512, 1024, False), (1025, 1023, True), (1025, 1024, False),
+    (2, 2046, True), (130, 4000, True),
     (4097, 300, False), (20, MOST - 20, True)])
 def test_same_paths_as_the_other_builders(n_veh, n_rx, clustered):
     if not torch.cuda.is_available():
