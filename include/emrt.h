@@ -382,7 +382,9 @@ emrt_status emrt_refresh_schedule(emrt_scene sc, float *state, uint8_t *los_ref,
                                   emrt_stream s);
 
 typedef struct {
-  uint64_t segments[EMRT_MAX_DEPTH + 1]; /* closest-hit segments per bounce */
+  uint64_t segments[EMRT_MAX_DEPTH + 1]; /* ray segments per bounce (a chain's
+                                 last one counts too where no receiver can be
+                                 near it and its end is not looked for)     */
   uint64_t candidates;        /* reception-sphere detections                 */
   uint64_t unique_candidates; /* after deduplication                         */
   uint64_t accepted;          /* paths written                                */

@@ -77,6 +77,24 @@ def test_records_are_the_candidates_in_canonical_order(engine, n_rx, n_tx, n_ray
     assert np.array_equal(kept, valid)
 
 
+def test_more_pairs_than_one_scan_takes(engine):
+    """16 x 70000 pairs (above 2^20: scanned by the general scan) against each
+    of two transmitters traced alone (70000 pairs)."""
+    sc, fr = _scene(70_000, 16)
+    g = engine.Scene(sc)
+    g.update(fr)
+    kw = dict(n_rays=20_000, max_depth=0)
+    whole = g.trace(**kw).records()
+    assert len(whole) > 1000
+    for t in (0, 11):
+        one = dataclasses.replace(fr, tx_pos=fr.tx_pos[t:t + 1], tx_vel=fr.tx_vel[t:t + 1])
+        g.update(one)
+        alone = g.trace(**kw).records()
+        part = whole[whole[:, 0] == t].copy()
+        part[:, 0] = 0
+        assert len(alone) > 100 and np.array_equal(alone, part)
+
+
 def test_a_pair_with_many_candidates(engine):
     """40 receivers in one place and few, wide rays: pairs of hundreds of
     candidates of many paths; the oracle's deduplication of the same records."""
