@@ -257,14 +257,19 @@ constexpr double kMargin = 1e-4;
 // inface_margin() of a reflection point P, as far as acceptance asks: whether
 // it is negative (outside the face) and whether it lies within kMargin of zero.
 // A warp issues an FP64 instruction every 64 cycles on GB300 and the margin
-// takes about 39 of them an edge, so the edges are first measured in FP32, in
-// coordinates from the face's first vertex (the difference taken in FP64):
-// with M the largest |P - a0| + |a - a0|, the FP32 distance is off by at most
-// about 13 x 2^-24 M (rounding of the three differences, of a cross and a dot
-// product and of one reciprocal root); a point whose distances all clear
-// kMargin by 2e-6 M (33 x 2^-24) on one side is decided, any other goes to the
-// FP64 margin.  Geometry of the city's 16k candidates 55 -> 24 us, of the
-// district's 3.7k 30 -> 20, of the toy scene's 38 19 -> 9.
+// takes about 39 of them an edge, so the edges are first measured in FP32: the
+// point in coordinates from the face's first vertex (the difference taken in
+// FP64), an edge as the difference of its stored ends, whose rounding is
+// relative to the edge (of ends rounded relative to the first vertex it would
+// be relative to them, and the distance off by M / |edge| times as much).  With
+// u = 2^-24 and M the largest |P - a0|_1 + |a - a0|_1, the distance is off by
+// at most 18 u M to first order: P - a rounded three times 2, the edge 1.4,
+// two products and a difference a component of the cross product 2.9, the
+// normal 1, the dot product 3, the reciprocal root (2 ulp) of the edge's
+// square 7.5.  A point whose distances all clear kMargin by 2e-6 M (33 u) on one
+// side is decided; any other, and a face with an edge whose square could leave
+// FP32's range, goes to the FP64 margin.  Geometry of the city's 16k candidates
+// 55 -> 24 us, of the district's 3.7k 30 -> 20, of the toy scene's 38 19 -> 9.
 struct InFace {
   bool outside, marginal;
 };
@@ -276,21 +281,26 @@ __device__ inline InFace inface(const GeomView &g, uint32_t f, D3 P, D3 n) {
     const float3 p = make_float3((float)p64.x, (float)p64.y, (float)p64.z);
     const float3 nf = make_float3((float)n.x, (float)n.y, (float)n.z);
     const float pl = fabsf(p.x) + fabsf(p.y) + fabsf(p.z);
-    float m = 1e30f, M = pl;
-    float3 a = f3(g.face_vert[info.x + info.y - 1]) - a0;
+    float m = 1e30f, M = pl, shortest = 1e30f;
+    float3 sa = f3(g.face_vert[info.x + info.y - 1]), a = sa - a0;
 #pragma unroll 4
     for (uint32_t k = 0; k < info.y; k++) {
-      const float3 b = f3(g.face_vert[info.x + k]) - a0;
-      const float3 e = b - a, w = p - a;
+      const float3 sb = f3(g.face_vert[info.x + k]);
+      const float3 b = sb - a0, e = sb - sa, w = p - a;
       const float3 c = make_float3(e.y * w.z - e.z * w.y, e.z * w.x - e.x * w.z,
                                    e.x * w.y - e.y * w.x);
-      m = fminf(m, dot3(c, nf) * rsqrtf(dot3(e, e)));
+      const float ee = dot3(e, e);
+      m = fminf(m, dot3(c, nf) * rsqrtf(ee));
       M = fmaxf(M, pl + (fabsf(b.x) + fabsf(b.y) + fabsf(b.z)));
+      shortest = fminf(shortest, ee);
+      sa = sb;
       a = b;
     }
     const float slack = (float)kMargin + 2e-6f * M;
-    if (m > slack) return InFace{false, false};
-    if (m < -slack) return InFace{true, false};
+    if (shortest > 1e-24f && M < 1e12f) {
+      if (m > slack) return InFace{false, false};
+      if (m < -slack) return InFace{true, false};
+    }
   }
   const double m = inface_margin(g, f, P, n);
   return InFace{m < 0.0, fabs(m) < kMargin};
