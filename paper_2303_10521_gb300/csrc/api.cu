@@ -915,8 +915,7 @@ emrt_status emrt_channel_backward_noalloc(emrt_scene s, const emrt_paths *paths,
 emrt_status emrt_channel_correlation(const double *h, uint32_t n_frames, uint32_t n_pairs,
                                      uint32_t max_lag, double *R, emrt_stream stream) {
   if (!h || !R || n_frames == 0 || n_pairs == 0) return EMRT_ERR_INVALID_ARG;
-  launch_correlation(h, n_frames, n_pairs, max_lag, R, (cudaStream_t)stream);
-  CK(cudaGetLastError());
+  CK(launch_correlation(h, n_frames, n_pairs, max_lag, R, (cudaStream_t)stream));
   return EMRT_OK;
 }
 

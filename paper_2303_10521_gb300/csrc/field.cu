@@ -886,17 +886,23 @@ __global__ void k_compact_ids(const uint32_t *flag, const uint32_t *pos, uint32_
 
 }  // namespace
 
-void launch_correlation(const double *h, uint32_t n_frames, uint32_t n_pairs, uint32_t max_lag,
-                        double *R, cudaStream_t s) {
+cudaError_t launch_correlation(const double *h, uint32_t n_frames, uint32_t n_pairs,
+                               uint32_t max_lag, double *R, cudaStream_t s) {
   // whole series in shared memory up to 96 KB a block (two blocks an SM)
   const bool whole = n_frames <= kCorrResident;
   const uint32_t n_buf = whole ? n_frames : kCorrChunk;
   const size_t smem = sizeof(double) * kCorrPairs * (whole ? n_buf : 2 * n_buf + kCorrLags);
   auto kern = whole ? k_correlation<true> : k_correlation<false>;
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the attribute is the function's for all threads of the process: always the
+  // largest size, so that no call lowers what another's launch needs
+  const size_t most =
+      sizeof(double) * kCorrPairs * (whole ? kCorrResident : 2 * kCorrChunk + kCorrLags);
+  const cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  if (e) return e;
   emrt::note_launch(), kern<<<ceil_div(n_pairs, kCorrPairs), kCorrBlock, smem, s>>>(
       h, n_frames, n_pairs, max_lag, n_buf, R);
+  return cudaGetLastError();
 }
 
 void launch_coherence(const GeomView &g, double freq, double r_thr, double *tc, cudaStream_t s) {

@@ -519,8 +519,11 @@ cudaError_t frame_trees_build(const FrameTreesBuf &f, BVHBuf &veh, BVHBuf &rx, B
   emrt::note_launch(), k_tree_blocks<<<blocks_total, kBlocksBlock, 0, s>>>(S);
   for (int k = 0; k < 3; k++) S.t[k].first = nodes_first[k];
   const size_t smem = sizeof(uint32_t) * round4(widest);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_tree_nodes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the attribute is the function's for all threads of the process: always the
+  // largest size, so that no build lowers what another's launch needs
+  const cudaError_t e = cudaFuncSetAttribute(k_tree_nodes, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(sizeof(uint32_t) * kFrameTreesMax));
+  if (e) return e;
   emrt::note_launch(), k_tree_nodes<<<nodes_total, kNodesBlock, smem, s>>>(S, mix.pad);
   return cudaGetLastError();
 }
