@@ -221,7 +221,8 @@ emrt_status emrt_rediscover(emrt_scene sc, const emrt_trace_params *p, emrt_path
  * as by emrt_trace (same record layout and canonical order; word 7 holds
  * the smallest backward ray index that found the path).
  * rx_ids: device uint32[n_ids] receiver indices to shoot from (distinct, each
- * < n_rx), or NULL for every receiver (n_ids ignored).  The ray ids pack
+ * < n_rx; an id that is not, of a list kept from a larger frame, gives no
+ * accepted path), or NULL for every receiver (n_ids ignored).  The ray ids pack
  * source << (32 - b) | ray index with b = bits(n_sources - 1), so the ray
  * count per receiver must be <= 2^(32 - b), and n_sources x count < 2^32;
  * otherwise EMRT_ERR_INVALID_ARG.  Capacity handling as emrt_trace. */

@@ -732,7 +732,7 @@ emrt_status emrt_trace_backward(emrt_scene s, const emrt_trace_params *p, const 
   GeomView gb = geom(s);
   if (rx_ids) {
     CK(grow(&s->src_pos, s->src_cap, n_src));
-    launch_gather_points(s->rx_pos, rx_ids, n_src, s->src_pos, st);
+    launch_gather_points(s->rx_pos, s->n_rx, rx_ids, n_src, s->src_pos, st);
     gb.tx_pos = s->src_pos;
   } else {
     gb.tx_pos = s->rx_pos;

@@ -61,8 +61,11 @@ __device__ inline uint32_t lower_bound(const uint32_t *rec, uint32_t n, const Pa
   return lo;
 }
 
+// A receiver id past the frame's (a source list of backward discovery kept from
+// a frame with more receivers) goes to the transmitter's last pair, behind that
+// pair's own records in the order; acceptance rejects it.
 __device__ inline uint32_t pair_of(const PairSpace &ps, uint32_t w0, uint32_t rx) {
-  if (!ps.tab) return w0 * ps.n_rx + rx;
+  if (!ps.tab) return w0 * ps.n_rx + min(rx, ps.n_rx - 1u);
   const BatchScene &t = ps.tab[w0 >> 8];
   return t.pair_begin + (w0 & 255u) * t.pair_rx + rx;
 }

@@ -512,9 +512,11 @@ __global__ void k_concat(const uint32_t *a, const uint32_t *na, uint32_t cap_a, 
 
 __global__ void k_set_u32(uint32_t *p, uint32_t v) { *p = v; }
 
-__global__ void k_gather_points(const float4 *pos, const uint32_t *ids, uint32_t n, float4 *out) {
+// an id past the n_pos points shoots from point 0 (its paths are rejected)
+__global__ void k_gather_points(const float4 *pos, uint32_t n_pos, const uint32_t *ids, uint32_t n,
+                                float4 *out) {
   uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) out[i] = pos[ids[i]];
+  if (i < n) out[i] = pos[ids[i] < n_pos ? ids[i] : 0u];
 }
 
 __global__ void k_reverse_cand(uint32_t *cand, const uint32_t *n, uint32_t cap,
@@ -763,9 +765,9 @@ void launch_merge_path(const KeyW<4> *keys, const uint32_t *vals, const uint32_t
 }
 void launch_set_u32(uint32_t *p, uint32_t v, cudaStream_t s) { emrt::note_launch(), k_set_u32<<<1, 1, 0, s>>>(p, v); }
 
-void launch_gather_points(const float4 *pos, const uint32_t *ids, uint32_t n, float4 *out,
-                          cudaStream_t s) {
-  if (n) emrt::note_launch(), k_gather_points<<<ceil_div(n, 256), 256, 0, s>>>(pos, ids, n, out);
+void launch_gather_points(const float4 *pos, uint32_t n_pos, const uint32_t *ids, uint32_t n,
+                          float4 *out, cudaStream_t s) {
+  if (n) emrt::note_launch(), k_gather_points<<<ceil_div(n, 256), 256, 0, s>>>(pos, n_pos, ids, n, out);
 }
 void launch_reverse_candidates(uint32_t *cand, const uint32_t *n, uint32_t cap,
                                const uint32_t *ids, cudaStream_t s) {

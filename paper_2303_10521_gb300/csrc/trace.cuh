@@ -153,9 +153,9 @@ void launch_merge_path(const KeyW<4> *keys, const uint32_t *vals, const uint32_t
 void launch_set_u32(uint32_t *p, uint32_t v, cudaStream_t s);
 
 // Backward tracing.  out[i] = pos[ids[i]] for i < n (source points of the
-// selected receivers).
-void launch_gather_points(const float4 *pos, const uint32_t *ids, uint32_t n, float4 *out,
-                          cudaStream_t s);
+// selected receivers; pos[0] for an id that is none of the n_pos points).
+void launch_gather_points(const float4 *pos, uint32_t n_pos, const uint32_t *ids, uint32_t n,
+                          float4 *out, cudaStream_t s);
 // Candidates found from the receiver side (word 0 = source index, word 1 =
 // transmitter, faces in the order met from the receiver) rewritten in place
 // in forward orientation: word 0 = transmitter, word 1 = ids[source] (or the
