@@ -141,16 +141,12 @@ cudaError_t ensure_cand(emrt_scene_s *s, uint64_t need) {
   return cudaSuccess;
 }
 
-// The pair counts, for n pairs (zeroed by each trace).
-cudaError_t ensure_pairs(emrt_scene_s *s, uint64_t n) {
-  if (n <= s->pair_cap && s->pair_count) return cudaSuccess;
-  uint64_t c = 0;
-  cudaError_t e;
-  s->pair_cap = 0;
-  e = grow(&s->pair_count, c, pair_words(n)); if (e) return e; c = 0;
-  e = grow(&s->pair_off, c, n + 4); if (e) return e;
-  s->pair_cap = n;
-  return cudaSuccess;
+// The pairs of n_tx transmitters and n_rx receivers.
+PairSpace pair_space(uint32_t n_tx, uint32_t n_rx) {
+  uint32_t shift = 0;
+  while ((uint64_t)n_tx * pair_lists(n_rx, shift) > kPairsMost) shift++;
+  const uint32_t per_tx = pair_lists(n_rx, shift);
+  return PairSpace{nullptr, n_rx, per_tx, shift, n_tx * per_tx};
 }
 
 emrt_status check_paths(const emrt_paths *p) {
@@ -224,6 +220,11 @@ emrt_status emrt_scene_create(const emrt_scene_desc *d, emrt_stream stream, emrt
   if (s->Fs) emrt::note_launch(), k_faces<<<ceil_div(s->Fs, 128), 128, 0, st>>>(d->face_off, d->face_xyz, d->face_mat,
                                                           s->Fs, s->face_plane, s->face_nf, s->face_info,
                                                           s->face_vert);
+  // any frame's pairs, so that no trace allocates for them (a captured one
+  // could not)
+  const uint64_t pairs = std::min<uint64_t>((uint64_t)s->max_tx * s->max_rx, kPairsMost);
+  if ((e = grow(&s->pair_count, c, pair_words(pairs)))) return fail(e); c = 0;
+  if ((e = grow(&s->pair_off, c, pairs + 4))) return fail(e); c = 0;
   if ((e = grow(&s->ctr, c, 1))) return fail(e); c = 0;
   if ((e = grow(&s->hist, c, 256 * kPrimGrid + 1))) return fail(e); c = 0;
   for (int k = 0; k < 2; k++) {
@@ -539,9 +540,8 @@ emrt_status run_trace(emrt_scene_s *s, const emrt_trace_params *p, uint64_t coun
   // candidate scratch
   want = merge_cache ? want + out->capacity : std::max<uint64_t>(want, out->capacity);
   CK(ensure_cand(s, want));
-  const uint32_t n_pairs = s->n_tx * s->n_rx;
-  CK(ensure_pairs(s, n_pairs));
-  cudaMemsetAsync(s->pair_count, 0, sizeof(uint32_t) * pair_words(n_pairs), st);
+  const PairSpace pairs = pair_space(s->n_tx, s->n_rx);
+  cudaMemsetAsync(s->pair_count, 0, sizeof(uint32_t) * pair_words(pairs.n_pairs), st);
   // counters: keep the error word, clear the rest
   cudaMemsetAsync(reinterpret_cast<char *>(c) + sizeof(uint32_t), 0,
                   sizeof(Counters) - sizeof(uint32_t), st);
@@ -641,8 +641,8 @@ emrt_status run_trace(emrt_scene_s *s, const emrt_trace_params *p, uint64_t coun
   s->ev_bounces = nev;
   cudaEventRecord(s->ev[1], st);
   if (backward) launch_reverse_candidates(s->cand, &c->n_cand, s->cand_cap, rx_ids, st);
-  launch_dedup(s->cand, &c->n_cand, s->cand_cap, PairSpace{nullptr, s->n_rx, n_pairs},
-               pair_bufs(s->pair_count, s->pair_off, n_pairs), s->uniq, s->pos, c, s->partial, st);
+  launch_dedup(s->cand, &c->n_cand, s->cand_cap, pairs,
+               pair_bufs(s->pair_count, s->pair_off, pairs.n_pairs), s->uniq, s->pos, c, st);
   cudaEventRecord(s->ev[2], st);
   if (merge_cache) {
     if (merge_after)  // the cache's revalidation on the side stream

@@ -37,7 +37,7 @@ struct emrt_batch_s {
   uint32_t *cand = nullptr, *uniq = nullptr, *pos = nullptr;
   float4 *apts = nullptr;  // acceptance scratch (reflection points)
   uint32_t *pair_count = nullptr, *pair_off = nullptr;  // candidates of every (scene, tx, rx)
-  uint32_t n_pairs = 0;
+  uint32_t n_pairs = 0, pair_shift = 0;  // see PairSpace
   Counters *ctr = nullptr;
   uint32_t *hist = nullptr, *partial = nullptr;
   int variant = default_bounce_variant();
@@ -132,8 +132,8 @@ void fill_table(emrt_batch_s *b) {
     t.out_count = b->outs[i].count;
     t.ends_last = walk_ends_last(b->total, t.g.n_rx, t.kappa);
     t.pair_begin = pairs;
-    t.pair_rx = s->max_rx;
-    pairs += b->n_tx[i] * s->max_rx;
+    t.pair_rx = pair_lists(s->max_rx, b->pair_shift);
+    pairs += b->n_tx[i] * t.pair_rx;
   }
 }
 
@@ -171,10 +171,10 @@ void enqueue(emrt_batch_s *b, int variant, bool sort_rays, cudaStream_t st) {
     launch_bounce_batched(variant, L, b->d_tab, b->n, st);
   }
   // canonical order (records carry the scene), accept, write to each scene
-  const PairSpace ps{b->d_tab, 0, b->n_pairs};
+  const PairSpace ps{b->d_tab, 0, 0, b->pair_shift, b->n_pairs};
   cudaMemsetAsync(b->pair_count, 0, sizeof(uint32_t) * pair_words(b->n_pairs), st);
   const PairBufs pairs = pair_bufs(b->pair_count, b->pair_off, b->n_pairs);
-  launch_dedup(b->cand, &c->n_cand, b->cand_cap, ps, pairs, b->uniq, b->pos, c, b->partial, st);
+  launch_dedup(b->cand, &c->n_cand, b->cand_cap, ps, pairs, b->uniq, b->pos, c, st);
   launch_accept_batched(b->d_tab, b->cand, &c->n_eff, c, b->apts, b->cand_cap, st);
   launch_keep(b->cand, &c->n_eff, KEEP_VALID, nullptr, 0, b->pos, &c->n_accepted, nullptr, c,
               b->partial, st);
@@ -244,7 +244,7 @@ emrt_status emrt_batch_create(const emrt_scene *scenes, uint32_t n, const emrt_t
   };
   b->n = n;
   uint32_t max_rx = 1, max_tx = 1, max_f = 1;
-  uint64_t tris = 0, n_pairs = 0;
+  uint64_t tris = 0;
   for (uint32_t i = 0; i < n; i++) {
     emrt_scene s = scenes[i];
     const emrt_trace_params &p = params[i];
@@ -264,7 +264,6 @@ emrt_status emrt_batch_create(const emrt_scene *scenes, uint32_t n, const emrt_t
     b->n_tx.push_back(s->n_tx);
     b->total += count * s->n_tx;
     b->Kmax = std::max(b->Kmax, p.max_depth);
-    n_pairs += (uint64_t)s->n_tx * s->max_rx;
     max_rx = std::max(max_rx, s->max_rx);
     max_tx = std::max(max_tx, s->n_tx);
     max_f = std::max(max_f, s->Fs + 6 * s->V + 1);
@@ -278,9 +277,15 @@ emrt_status emrt_batch_create(const emrt_scene *scenes, uint32_t n, const emrt_t
   BCK(cudaMalloc(&b->ctr, sizeof(Counters)));
   BCK(cudaMalloc(&b->hist, sizeof(uint32_t) * (256 * kPrimGrid + 1)));
   BCK(cudaMalloc(&b->partial, sizeof(uint32_t) * (kPrimGrid + 1)));
-  b->n_pairs = (uint32_t)n_pairs;
-  BCK(cudaMalloc(&b->pair_count, sizeof(uint32_t) * pair_words(n_pairs)));
-  BCK(cudaMalloc(&b->pair_off, sizeof(uint32_t) * (n_pairs + 4)));
+  auto pairs = [&](uint32_t shift) {
+    uint64_t p = 0;
+    for (uint32_t i = 0; i < n; i++) p += (uint64_t)b->n_tx[i] * pair_lists(scenes[i]->max_rx, shift);
+    return p;
+  };
+  while (pairs(b->pair_shift) > kPairsMost) b->pair_shift++;
+  b->n_pairs = (uint32_t)pairs(b->pair_shift);
+  BCK(cudaMalloc(&b->pair_count, sizeof(uint32_t) * pair_words(b->n_pairs)));
+  BCK(cudaMalloc(&b->pair_off, sizeof(uint32_t) * (b->n_pairs + 4)));
   BCK(cudaMemsetAsync(b->ctr, 0, sizeof(Counters), st));
   // direction tables, shared between scenes with the same ray set
   KeyW<1> *k0 = nullptr;

@@ -65,9 +65,9 @@ __device__ inline uint32_t lower_bound(const uint32_t *rec, uint32_t n, const Pa
 // a frame with more receivers) goes to the transmitter's last pair, behind that
 // pair's own records in the order; acceptance rejects it.
 __device__ inline uint32_t pair_of(const PairSpace &ps, uint32_t w0, uint32_t rx) {
-  if (!ps.tab) return w0 * ps.n_rx + min(rx, ps.n_rx - 1u);
+  if (!ps.tab) return w0 * ps.per_tx + (min(rx, ps.n_rx - 1u) >> ps.shift);
   const BatchScene &t = ps.tab[w0 >> 8];
-  return t.pair_begin + (w0 & 255u) * t.pair_rx + rx;
+  return t.pair_begin + (w0 & 255u) * t.pair_rx + (rx >> ps.shift);
 }
 
 // place of every candidate within its pair, in order of arrival; group[g]:
@@ -406,16 +406,11 @@ PairBufs pair_bufs(uint32_t *count, uint32_t *off, uint64_t n_pairs) {
 
 void launch_dedup(uint32_t *cand, const uint32_t *n_cand, uint32_t cap, const PairSpace &ps,
                   const PairBufs &pb, uint32_t *lists, uint32_t *place, Counters *ctr,
-                  uint32_t *partial, cudaStream_t s) {
+                  cudaStream_t s) {
   emrt::note_launch(), k_pair_count<<<kPathsGrid, kPathsBlock, 0, s>>>(cand, n_cand, cap, ps, pb.count, pb.group, place,
                                                                      ctr);
-  if (ps.n_pairs <= kPairScanMax) {
-    emrt::note_launch(), k_pair_scan<<<ceil_div(ps.n_pairs, kPairGroup), kScanBlock, 0, s>>>(pb.count, pb.group,
-                                                                                        ps.n_pairs, pb.off);
-  } else {
-    launch_set_u32(&ctr->tmp, ps.n_pairs, s);
-    exclusive_scan(&ctr->tmp, pb.count, pb.off, pb.off + ps.n_pairs, partial, s);
-  }
+  emrt::note_launch(), k_pair_scan<<<ceil_div(ps.n_pairs, kPairGroup), kScanBlock, 0, s>>>(pb.count, pb.group,
+                                                                                      ps.n_pairs, pb.off);
   emrt::note_launch(), k_pair_place<<<kPathsGrid, kPathsBlock, 0, s>>>(cand, &ctr->n_eff, ps, pb.off, place, lists);
   emrt::note_launch(), k_pair_order<<<kPathsGrid, kPathsBlock, 0, s>>>(lists, &ctr->n_eff, ps, pb.off, cand, ctr);
 }

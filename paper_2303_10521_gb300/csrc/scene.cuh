@@ -57,9 +57,8 @@ struct emrt_scene_s {
   float4 *apts = nullptr;  // acceptance scratch: reflection points, point-major
   KeyW<4> *keys[2] = {nullptr, nullptr};
   uint32_t *vals[2] = {nullptr, nullptr};
-  // candidates of every (tx, rx) pair: counts and places (max_tx x max_rx)
+  // candidates of every (tx, rx) pair: counts and places, for any frame
   uint32_t *pair_count = nullptr, *pair_off = nullptr;
-  uint64_t pair_cap = 0;
   // adjoint scratch
   double *contrib = nullptr;
   uint64_t contrib_cap = 0;

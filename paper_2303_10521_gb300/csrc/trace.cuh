@@ -92,7 +92,7 @@ struct BatchScene {
   uint32_t *out_count;
   int ends_last;          // see walk_ends_last
   uint32_t pair_begin;    // first pair of this scene in the batch's pair space
-  uint32_t pair_rx;       // its receiver capacity (pairs of a transmitter)
+  uint32_t pair_rx;       // pairs of a transmitter, for its receiver capacity
 };
 constexpr uint32_t kBatchMaxScenes = 64, kBatchMaxTx = 16, kBatchMaxCount = 1u << 22;
 
@@ -166,13 +166,20 @@ void launch_reverse_candidates(uint32_t *cand, const uint32_t *n, uint32_t cap,
 
 // ---------------------------------------------------------------------------
 // Path records after discovery (paths.cu).
-// The (tx, rx) pairs candidates belong to: pair tx * n_rx + rx of one scene,
-// or the scenes' ranges of a batch's table.
+// The (tx, rx) pairs candidates belong to, counted and listed by pair: pair
+// tx * per_tx + (rx >> shift) of one scene, or the scenes' ranges of a batch's
+// table.  shift: with more than kPairsMost pairs 2^shift neighbouring receivers
+// share a list (the order within a list compares the receivers too), so that
+// the counts have a fixed size and one block sums the groups before its own
+// (4096 words).
 struct PairSpace {
   const BatchScene *tab;  // null: one scene
-  uint32_t n_rx, n_pairs;
+  uint32_t n_rx, per_tx, shift, n_pairs;
 };
 constexpr uint32_t kPairGroup = 256;  // pairs counted together once more
+constexpr uint32_t kPairsMost = 1u << 20;
+// lists a transmitter of n_rx > 0 receivers
+inline uint32_t pair_lists(uint32_t n_rx, uint32_t shift) { return ((n_rx - 1u) >> shift) + 1u; }
 struct PairBufs {
   uint32_t *count;  // [n_pairs up to a multiple of 4], zero before a dedup, as
   uint32_t *group;  // [n_pairs / kPairGroup rounded up]
@@ -181,8 +188,6 @@ struct PairBufs {
 // words at count for n_pairs pairs (count, then group), and their places
 uint64_t pair_words(uint64_t n_pairs);
 PairBufs pair_bufs(uint32_t *count, uint32_t *off, uint64_t n_pairs);
-// pairs up to which a group's block sums the groups before it (4096 words)
-constexpr uint32_t kPairScanMax = 1u << 20;
 // min(*n_cand, cap) candidates at cand, in place, to canonical order; equal
 // paths become one record with the smallest ray index and duplicates behind
 // it, whose depth (word 2) is no path's.  ctr->n_eff: records, duplicates
@@ -190,7 +195,7 @@ constexpr uint32_t kPairScanMax = 1u << 20;
 // scratch of cap records and cap words.
 void launch_dedup(uint32_t *cand, const uint32_t *n_cand, uint32_t cap, const PairSpace &ps,
                   const PairBufs &pb, uint32_t *lists, uint32_t *place, Counters *ctr,
-                  uint32_t *partial, cudaStream_t s);
+                  cudaStream_t s);
 enum KeepWhich { KEEP_VALID, KEEP_PATHS, KEEP_ALL };  // valid; not a duplicate; every record
 // The kept ones of *n records in order to out (at most cap; more raise
 // ERR_PATH_OVERFLOW), their number to *total and *count (may be null); with
