@@ -124,6 +124,7 @@ void launch_evicted(const Counters *c, uint32_t *out, cudaStream_t s) {
 
 cudaError_t ensure_cand(emrt_scene_s *s, uint64_t need) {
   if (need <= s->cand_cap && s->cand) return cudaSuccess;
+  s->cand_cap = 0;
   uint64_t c = 0;
   cudaError_t e;
   uint64_t cap = std::max<uint64_t>(need, 1024);
@@ -137,6 +138,8 @@ cudaError_t ensure_cand(emrt_scene_s *s, uint64_t need) {
     e = grow(&s->keys[k], c, cap); if (e) return e; c = 0;
     e = grow(&s->vals[k], c, cap); if (e) return e; c = 0;
   }
+  e = grow(&s->pair_table, c, pair_slots(cap)); if (e) return e;
+  e = zero_table(s->pair_table, cap); if (e) return e;
   s->cand_cap = (uint32_t)cap;
   return cudaSuccess;
 }
@@ -322,7 +325,7 @@ void emrt_scene_destroy(emrt_scene s) {
   for (int k = 0; k < 2; k++) { cudaFree(s->rkeys[k]); cudaFree(s->rvals[k]); }
   cudaFree(s->cand); cudaFree(s->uniq); cudaFree(s->head); cudaFree(s->pos); cudaFree(s->apts);
   for (int k = 0; k < 2; k++) { cudaFree(s->keys[k]); cudaFree(s->vals[k]); }
-  cudaFree(s->pair_count); cudaFree(s->pair_off);
+  cudaFree(s->pair_count); cudaFree(s->pair_off); cudaFree(s->pair_table);
   cudaFree(s->contrib);
   for (int k = 0; k < 4; k++)
     if (s->ev[k]) cudaEventDestroy(s->ev[k]);
@@ -642,7 +645,8 @@ emrt_status run_trace(emrt_scene_s *s, const emrt_trace_params *p, uint64_t coun
   cudaEventRecord(s->ev[1], st);
   if (backward) launch_reverse_candidates(s->cand, &c->n_cand, s->cand_cap, rx_ids, st);
   launch_dedup(s->cand, &c->n_cand, s->cand_cap, pairs,
-               pair_bufs(s->pair_count, s->pair_off, pairs.n_pairs), s->uniq, s->pos, c, st);
+               pair_bufs(s->pair_count, s->pair_off, pairs.n_pairs), s->uniq, s->pos, s->pair_table,
+               c, st);
   cudaEventRecord(s->ev[2], st);
   if (merge_cache) {
     if (merge_after)  // the cache's revalidation on the side stream

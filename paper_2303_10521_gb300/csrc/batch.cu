@@ -37,6 +37,7 @@ struct emrt_batch_s {
   uint32_t *cand = nullptr, *uniq = nullptr, *pos = nullptr;
   float4 *apts = nullptr;  // acceptance scratch (reflection points)
   uint32_t *pair_count = nullptr, *pair_off = nullptr;  // candidates of every (scene, tx, rx)
+  uint32_t *pair_table = nullptr;
   uint32_t n_pairs = 0, pair_shift = 0;  // see PairSpace
   Counters *ctr = nullptr;
   uint32_t *hist = nullptr, *partial = nullptr;
@@ -64,7 +65,8 @@ emrt_status st_of(cudaError_t e) {
 
 void free_scratch(emrt_batch_s *b) {
   cudaFree(b->cand); cudaFree(b->uniq); cudaFree(b->pos); cudaFree(b->apts);
-  b->cand = b->uniq = b->pos = nullptr;
+  cudaFree(b->pair_table);
+  b->cand = b->uniq = b->pos = b->pair_table = nullptr;
   b->apts = nullptr;
   b->cand_cap = 0;
 }
@@ -77,6 +79,8 @@ cudaError_t alloc_cand(emrt_batch_s *b, uint64_t cap) {
   if ((e = cudaMalloc(&b->uniq, 32 * cap))) return e;
   if ((e = cudaMalloc(&b->pos, 4 * cap))) return e;
   if ((e = cudaMalloc(&b->apts, sizeof(float4) * (EMRT_MAX_DEPTH + 2) * cap))) return e;
+  if ((e = cudaMalloc(&b->pair_table, sizeof(uint32_t) * pair_slots(cap)))) return e;
+  if ((e = zero_table(b->pair_table, cap))) return e;
   b->cand_cap = (uint32_t)cap;
   return cudaSuccess;
 }
@@ -174,7 +178,7 @@ void enqueue(emrt_batch_s *b, int variant, bool sort_rays, cudaStream_t st) {
   const PairSpace ps{b->d_tab, 0, 0, b->pair_shift, b->n_pairs};
   cudaMemsetAsync(b->pair_count, 0, sizeof(uint32_t) * pair_words(b->n_pairs), st);
   const PairBufs pairs = pair_bufs(b->pair_count, b->pair_off, b->n_pairs);
-  launch_dedup(b->cand, &c->n_cand, b->cand_cap, ps, pairs, b->uniq, b->pos, c, st);
+  launch_dedup(b->cand, &c->n_cand, b->cand_cap, ps, pairs, b->uniq, b->pos, b->pair_table, c, st);
   launch_accept_batched(b->d_tab, b->cand, &c->n_eff, c, b->apts, b->cand_cap, st);
   launch_keep(b->cand, &c->n_eff, KEEP_VALID, nullptr, 0, b->pos, &c->n_accepted, nullptr, c,
               b->partial, st);

@@ -70,42 +70,96 @@ __device__ inline uint32_t pair_of(const PairSpace &ps, uint32_t w0, uint32_t rx
   return t.pair_begin + (w0 & 255u) * t.pair_rx + (rx >> ps.shift);
 }
 
-// place of every candidate within its pair, in order of arrival; group[g]:
-// candidates of pairs kPairGroup g .. kPairGroup (g + 1) - 1
-__global__ void __launch_bounds__(kPathsBlock) k_pair_count(const uint32_t *cand,
-                                                            const uint32_t *n_cand, uint32_t cap,
-                                                            PairSpace ps, uint32_t *count,
-                                                            uint32_t *group, uint32_t *place,
-                                                            Counters *ctr) {
-  const uint32_t n = min(*n_cand, cap);
-  uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) {
-    ctr->n_eff = n;
-    if (*n_cand > cap) atomicOr(&ctr->err, ERR_CAND_OVERFLOW);
+constexpr uint32_t kLeftOut = 0xffffffffu;  // place of a candidate left out
+
+__device__ inline uint64_t slot_of(const PathOrder &o, uint64_t slots) {
+  unsigned long long h = o.k0 * 0x9e3779b97f4a7c15ull;
+  h = (h ^ (h >> 32) ^ o.k1) * 0xd6e8feb86659fd93ull;
+  h = (h ^ (h >> 32) ^ o.k2) * 0x9e3779b97f4a7c15ull;
+  h = (h ^ (h >> 32) ^ o.k3) * 0xd6e8feb86659fd93ull;
+  return __umul64hi(h ^ (h >> 32), slots);
+}
+
+// Whether candidate i is the first of its path in the table; another lowers the
+// first one's ray index.  The table has more slots than there are candidates.
+__device__ inline bool first_met(uint32_t *cand, uint32_t i, uint32_t *table, uint64_t slots) {
+  const PathOrder o = order_at(cand, i);
+  uint64_t at = slot_of(o, slots);
+  for (uint64_t k = 0; k < slots; k++) {
+    uint32_t other = *reinterpret_cast<volatile uint32_t *>(table + at);
+    if (!other) other = atomicCAS(table + at, 0u, i + 1u);
+    if (!other) return true;
+    const uint32_t c = other - 1u;
+    if (same(order_at(cand, c), o)) {
+      const uint32_t ray = cand[8ull * i + 7];
+      if (ray < *reinterpret_cast<volatile uint32_t *>(cand + 8ull * c + 7))
+        atomicMin(cand + 8ull * c + 7, ray);
+      return false;
+    }
+    at = at + 1 == slots ? 0 : at + 1;
   }
-  for (; i < n; i += gridDim.x * blockDim.x) {
-    const uint32_t p = pair_of(ps, cand[8ull * i], cand[8ull * i + 1]);
-    place[i] = atomicAdd(count + p, 1u);
-    atomicAdd(group + p / kPairGroup, 1u);
+  return true;
+}
+
+// Takes candidate i, a first one, out of the table.  Others are taken out at the
+// same time, so an empty slot does not end the search.
+__device__ inline void take_out(const uint32_t *cand, uint32_t i, uint32_t *table, uint64_t slots) {
+  uint64_t at = slot_of(order_at(cand, i), slots);
+  for (uint64_t k = 0; k < slots; k++) {
+    uint32_t *t = table + at;
+    if (*reinterpret_cast<volatile uint32_t *>(t) == i + 1u) {
+      *t = 0u;
+      return;
+    }
+    at = at + 1 == slots ? 0 : at + 1;
   }
 }
 
-// off[p] = counts before pair p, off[n] = all: a block scans one group of
+// place of every candidate within its pair, in order of arrival; group[g]:
+// candidates of pairs kPairGroup g .. kPairGroup (g + 1) - 1
+__global__ void __launch_bounds__(kPathsBlock) k_pair_count(uint32_t *cand,
+                                                            const uint32_t *n_cand, uint32_t cap,
+                                                            PairSpace ps, PairBufs pb,
+                                                            uint32_t *place, uint32_t *table,
+                                                            uint64_t slots, Counters *ctr) {
+  const uint32_t n = min(*n_cand, cap);
+  uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0 && *n_cand > cap) atomicOr(&ctr->err, ERR_CAND_OVERFLOW);
+  for (; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t p = pair_of(ps, cand[8ull * i], cand[8ull * i + 1]);
+    uint32_t at = atomicAdd(pb.count + p, 1u);
+    if (at >= kPairLong)
+      at = first_met(cand, i, table, slots) ? kPairLong + atomicAdd(pb.more + p, 1u) : kLeftOut;
+    place[i] = at;
+    if (at != kLeftOut) atomicAdd(pb.group + p / kPairGroup, 1u);
+  }
+}
+
+// records of a pair's list
+__device__ inline uint32_t list_length(const PairBufs &pb, uint32_t p, uint32_t count) {
+  return count <= kPairLong ? count : kPairLong + pb.more[p];
+}
+
+// off[p] = records before pair p, off[n] and ctr->n_eff = all: a block scans one group of
 // pairs, four a thread (16-byte loads; count is zero up to the next multiple
 // of 4), after the sum of the groups before it.  One launch without a barrier:
 // 40000 pairs in 3.0 us, 13.9 with one block scanning them all.
 constexpr int kScanBlock = kPairGroup / 4;
-__global__ void __launch_bounds__(kScanBlock) k_pair_scan(const uint32_t *count,
-                                                           const uint32_t *group, uint32_t n,
-                                                           uint32_t *off) {
+__global__ void __launch_bounds__(kScanBlock) k_pair_scan(PairBufs pb, uint32_t n, Counters *ctr) {
   __shared__ uint32_t s_warp[kScanBlock / 32], s_base;
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t i = blockIdx.x * kScanBlock + threadIdx.x;  // of four pairs
   if (threadIdx.x == 0) s_base = 0;
   uint4 c = make_uint4(0u, 0u, 0u, 0u);
-  if (4 * i < n) c = reinterpret_cast<const uint4 *>(count)[i];
+  if (4 * i < n) {
+    c = reinterpret_cast<const uint4 *>(pb.count)[i];
+    c.x = list_length(pb, 4 * i, c.x);
+    c.y = list_length(pb, 4 * i + 1, c.y);
+    c.z = list_length(pb, 4 * i + 2, c.z);
+    c.w = list_length(pb, 4 * i + 3, c.w);
+  }
   uint32_t before = 0;
-  for (uint32_t g = threadIdx.x; g < blockIdx.x; g += kScanBlock) before += group[g];
+  for (uint32_t g = threadIdx.x; g < blockIdx.x; g += kScanBlock) before += pb.group[g];
   const uint32_t sum = c.x + c.y + c.z + c.w;
   uint32_t incl = sum;
   for (int o = 1; o < 32; o <<= 1) {
@@ -120,20 +174,25 @@ __global__ void __launch_bounds__(kScanBlock) k_pair_scan(const uint32_t *count,
   uint32_t run = s_base + incl - sum;
   for (uint32_t w = 0; w < warp; w++) run += s_warp[w];
   if (4 * i >= n) return;
-  reinterpret_cast<uint4 *>(off)[i] = make_uint4(run, run + c.x, run + c.x + c.y, run + c.x + c.y + c.z);
-  if (4 * i + 4 >= n) off[n] = run + sum;
+  reinterpret_cast<uint4 *>(pb.off)[i] = make_uint4(run, run + c.x, run + c.x + c.y, run + c.x + c.y + c.z);
+  if (4 * i + 4 >= n) pb.off[n] = ctr->n_eff = run + sum;
 }
 
-__global__ void __launch_bounds__(kPathsBlock) k_pair_place(const uint32_t *cand, const uint32_t *n,
+__global__ void __launch_bounds__(kPathsBlock) k_pair_place(const uint32_t *cand,
+                                                            const uint32_t *n_cand, uint32_t cap,
                                                             PairSpace ps, const uint32_t *off,
-                                                            const uint32_t *place, uint32_t *lists) {
-  const uint32_t cnt = *n;
+                                                            const uint32_t *place, uint32_t *lists,
+                                                            uint32_t *table, uint64_t slots) {
+  const uint32_t cnt = min(*n_cand, cap);
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += gridDim.x * blockDim.x) {
+    const uint32_t at = place[i];
+    if (at == kLeftOut) continue;
     const uint4 *r = reinterpret_cast<const uint4 *>(cand + 8ull * i);
     const uint4 a = r[0], b = r[1];
-    uint4 *o = reinterpret_cast<uint4 *>(lists + 8ull * (off[pair_of(ps, a.x, a.y)] + place[i]));
+    uint4 *o = reinterpret_cast<uint4 *>(lists + 8ull * (off[pair_of(ps, a.x, a.y)] + at));
     o[0] = a;
     o[1] = b;
+    if (at >= kPairLong) take_out(cand, i, table, slots);
   }
 }
 
@@ -398,20 +457,22 @@ constexpr int kPathsGrid = 4 * 152;
 }  // namespace
 
 uint64_t pair_words(uint64_t n_pairs) {
-  return (n_pairs + 3) / 4 * 4 + (n_pairs + kPairGroup - 1) / kPairGroup;
+  return 2 * ((n_pairs + 3) / 4 * 4) + (n_pairs + kPairGroup - 1) / kPairGroup;
 }
 PairBufs pair_bufs(uint32_t *count, uint32_t *off, uint64_t n_pairs) {
-  return PairBufs{count, count + (n_pairs + 3) / 4 * 4, off};
+  const uint64_t n4 = (n_pairs + 3) / 4 * 4;
+  return PairBufs{count, count + n4, count + 2 * n4, off};
 }
 
 void launch_dedup(uint32_t *cand, const uint32_t *n_cand, uint32_t cap, const PairSpace &ps,
-                  const PairBufs &pb, uint32_t *lists, uint32_t *place, Counters *ctr,
-                  cudaStream_t s) {
-  emrt::note_launch(), k_pair_count<<<kPathsGrid, kPathsBlock, 0, s>>>(cand, n_cand, cap, ps, pb.count, pb.group, place,
+                  const PairBufs &pb, uint32_t *lists, uint32_t *place, uint32_t *table,
+                  Counters *ctr, cudaStream_t s) {
+  const uint64_t slots = pair_slots(cap);
+  emrt::note_launch(), k_pair_count<<<kPathsGrid, kPathsBlock, 0, s>>>(cand, n_cand, cap, ps, pb, place, table, slots,
                                                                      ctr);
-  emrt::note_launch(), k_pair_scan<<<ceil_div(ps.n_pairs, kPairGroup), kScanBlock, 0, s>>>(pb.count, pb.group,
-                                                                                      ps.n_pairs, pb.off);
-  emrt::note_launch(), k_pair_place<<<kPathsGrid, kPathsBlock, 0, s>>>(cand, &ctr->n_eff, ps, pb.off, place, lists);
+  emrt::note_launch(), k_pair_scan<<<ceil_div(ps.n_pairs, kPairGroup), kScanBlock, 0, s>>>(pb, ps.n_pairs, ctr);
+  emrt::note_launch(), k_pair_place<<<kPathsGrid, kPathsBlock, 0, s>>>(cand, n_cand, cap, ps, pb.off, place, lists,
+                                                                     table, slots);
   emrt::note_launch(), k_pair_order<<<kPathsGrid, kPathsBlock, 0, s>>>(lists, &ctr->n_eff, ps, pb.off, cand, ctr);
 }
 

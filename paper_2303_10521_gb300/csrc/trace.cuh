@@ -182,20 +182,35 @@ constexpr uint32_t kPairsMost = 1u << 20;
 inline uint32_t pair_lists(uint32_t n_rx, uint32_t shift) { return ((n_rx - 1u) >> shift) + 1u; }
 struct PairBufs {
   uint32_t *count;  // [n_pairs up to a multiple of 4], zero before a dedup, as
+  uint32_t *more;   // [the same], distinct ones past kPairLong, and
   uint32_t *group;  // [n_pairs / kPairGroup rounded up]
   uint32_t *off;    // [n_pairs + 4]
 };
-// words at count for n_pairs pairs (count, then group), and their places
+// Candidates of a pair past the first kPairLong are looked up in a table of
+// those already met (open addressing, 0 empty, else candidate index + 1) and
+// leave out what it holds: ordering a list takes its length squared compares,
+// and a receiver at a transmitter's own position is met by every primary ray
+// (100k of them: trace 22 ms with the whole list ordered, 0.21 so).
+// The table has pair_slots(cap) words, zero before and after every dedup.
+constexpr uint32_t kPairLong = 256;
+inline uint64_t pair_slots(uint64_t cap) { return 2 * cap; }
+// a new table's zeros (when it returns they are there for every stream)
+inline cudaError_t zero_table(uint32_t *table, uint64_t cap) {
+  const cudaError_t e = cudaMemset(table, 0, sizeof(uint32_t) * pair_slots(cap));
+  return e ? e : cudaStreamSynchronize(nullptr);
+}
+// words at count for n_pairs pairs (count, more, group), and their places
 uint64_t pair_words(uint64_t n_pairs);
 PairBufs pair_bufs(uint32_t *count, uint32_t *off, uint64_t n_pairs);
 // min(*n_cand, cap) candidates at cand, in place, to canonical order; equal
 // paths become one record with the smallest ray index and duplicates behind
-// it, whose depth (word 2) is no path's.  ctr->n_eff: records, duplicates
-// included; ctr->n_unique is raised by the others (0 before).  lists, place:
-// scratch of cap records and cap words.
+// it, whose depth (word 2) is no path's (those left out above are not among
+// them).  ctr->n_eff: records, duplicates included; ctr->n_unique is raised by
+// the others (0 before).  lists, place: scratch of cap records and cap words;
+// table: pair_slots(cap) words.
 void launch_dedup(uint32_t *cand, const uint32_t *n_cand, uint32_t cap, const PairSpace &ps,
-                  const PairBufs &pb, uint32_t *lists, uint32_t *place, Counters *ctr,
-                  cudaStream_t s);
+                  const PairBufs &pb, uint32_t *lists, uint32_t *place, uint32_t *table,
+                  Counters *ctr, cudaStream_t s);
 enum KeepWhich { KEEP_VALID, KEEP_PATHS, KEEP_ALL };  // valid; not a duplicate; every record
 // The kept ones of *n records in order to out (at most cap; more raise
 // ERR_PATH_OVERFLOW), their number to *total and *count (may be null); with
