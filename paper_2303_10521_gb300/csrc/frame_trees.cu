@@ -95,28 +95,88 @@ __global__ void __launch_bounds__(kBinsBlock) k_tree_bins(FrameTreesView T) {
   T.member[s_first[code >> kTreeBinShift] + T.slot[p]] = make_uint2(code, p);
 }
 
+// (code, primitive): equal codes are ordered by index
+__device__ inline uint64_t order_key(uint2 m) { return (uint64_t)m.x << 32 | m.y; }
+
 // One thread a list place (a warp's threads mostly share their bin, whose
 // list they read together): smaller keys of the bin, of both classes and of
-// its own, and the leaf written in its places.
-constexpr int kRankBlock = 128;
+// its own, and the leaf written in its places.  A bin of more than kRankLong
+// primitives (a crowd on one square) is not compared all with all: the block
+// orders its own places of the bin, every member finds where it stands among
+// them (8 steps) and is counted there, and a place's rank is the sum of the
+// counts up to it.  Update with every receiver within 100 m: 4000 225 -> 42 us,
+// 15000 770 -> 66, 32700 1650 -> 112 (spread over 2 km: 31, 37, 56); blocks of
+// 128 places 155 at 32700, of 512 118.
+constexpr int kRankBlock = 256;
+constexpr uint32_t kRankLong = 256;
+static_assert(kRankLong >= kRankBlock, "only the bins at a block's two ends can be long");
 __global__ void __launch_bounds__(kRankBlock) k_tree_rank(FrameTreesView T) {
-  const uint32_t i = blockIdx.x * kRankBlock + threadIdx.x;
-  if (i >= T.V + T.R) return;
-  const uint2 me = T.member[i];
+  __shared__ uint64_t s_own[kRankBlock], s_key[kRankBlock];
+  __shared__ uint32_t s_hist[kRankBlock];
+  const uint32_t n = T.V + T.R, i0 = blockIdx.x * kRankBlock, i = i0 + threadIdx.x;
+  const bool live = i < n;
+  const uint2 me = T.member[min(i, n - 1u)];
   const uint32_t p = me.y, bin = me.x >> kTreeBinShift;
   const bool veh = p < T.V;
   const uint32_t b0 = T.first[bin], b1 = T.first[bin + 1], v0 = T.first_v[bin];
   const float4 a = veh ? T.veh_lo[p] : T.rx[p - T.V], b = veh ? T.veh_hi[p] : a;
-  uint32_t mix = 0, vehs = 0;
+  // places before this one in its bin: all in the low half, vehicles in the high
+  uint32_t rank = 0;
+  static_assert(kFrameTreesMax < 65536u, "two counts a word");
+  const bool is_long = live && b1 - b0 > kRankLong;
+  if (live && !is_long) {
 #pragma unroll 4
-  for (uint32_t q = b0; q < b1; q++) {
-    const uint2 m = T.member[q];
-    const bool less = m.x < me.x || (m.x == me.x && m.y < p);  // equal codes by index
-    mix += less ? 1u : 0u;
-    vehs += less && m.y < T.V ? 1u : 0u;
+    for (uint32_t q = b0; q < b1; q++) {
+      const uint2 m = T.member[q];
+      if (order_key(m) < order_key(me)) rank += m.y < T.V ? 0x10001u : 1u;
+    }
   }
-  const uint32_t own = veh ? v0 + vehs : b0 - v0 + mix - vehs;
-  mix += b0;
+  if (__syncthreads_or(is_long)) {
+    s_own[threadIdx.x] = order_key(me);
+    uint32_t done = 0xffffffffu;  // bin of the first round
+    for (int end = 0; end < 2; end++) {
+      const uint32_t e = T.member[end ? min(i0 + kRankBlock, n) - 1u : i0].x >> kTreeBinShift;
+      const uint32_t e0 = T.first[e], e1 = T.first[e + 1];
+      if (e == done || e1 - e0 <= kRankLong) continue;  // the same for the whole block
+      done = e;
+      const uint32_t q0 = max(e0, i0) - i0, q1 = min(e1, i0 + kRankBlock) - i0;
+      const bool mine = live && bin == e;
+      s_key[threadIdx.x] = ~0ull;
+      s_hist[threadIdx.x] = 0u;
+      __syncthreads();
+      uint32_t at = 0;  // order among the block's own
+      for (uint32_t q = q0; q < q1; q++) at += s_own[q] < s_own[threadIdx.x] ? 1u : 0u;
+      if (mine) s_key[at] = s_own[threadIdx.x];
+      __syncthreads();
+      uint32_t first = 0;
+#pragma unroll 4
+      for (uint32_t q = e0 + threadIdx.x; q < e1; q += kRankBlock) {
+        const uint2 m = T.member[q];
+        const uint64_t k = order_key(m);
+        const uint32_t one = m.y < T.V ? 0x10001u : 1u;
+        uint32_t above = 0;  // own keys up to k, the last not counted
+#pragma unroll
+        for (uint32_t s = kRankBlock / 2; s; s >>= 1)
+          if (s_key[above + s - 1] <= k) above += s;
+        if (!above) {
+          first += one;
+        } else {
+          if (s_key[above] <= k) above++;
+          if (above < q1 - q0) atomicAdd(&s_hist[above], one);
+        }
+      }
+      for (int o = 16; o; o >>= 1) first += __shfl_xor_sync(0xffffffffu, first, o);
+      if ((threadIdx.x & 31) == 0 && first) atomicAdd(&s_hist[0], first);
+      __syncthreads();
+      if (mine)
+        for (uint32_t q = 0; q <= at; q++) rank += s_hist[q];
+      __syncthreads();
+    }
+  }
+  if (!live) return;
+  const uint32_t vehs = rank >> 16, all = rank & 0xffffu;
+  const uint32_t own = veh ? v0 + vehs : b0 - v0 + all - vehs;
+  const uint32_t mix = b0 + all;
   T.prims[2][2ull * mix] = make_float4(a.x, a.y, a.z, __uint_as_float(p));
   T.prims[2][2ull * mix + 1] = make_float4(b.x, b.y, b.z, 0.f);
   T.sorted[2][mix] = me.x;
@@ -317,6 +377,35 @@ struct SmallShared {
 };
 static_assert(kTreeBins == 4 * kSmallBlock, "four bins a thread");
 
+// A bin of more than kSmallLong members: the block sorts all members (bitonic,
+// 66 steps of 2048 keys, a warp's own 64 places without block barriers) instead
+// of comparing the bin's with one another.  The sort adds 14 us to a 2048
+// frame's 29, whatever the bins; bins of 200 add 8 by comparing (the line lies
+// where the two meet), one bin of all 2000 added 154.
+constexpr uint32_t kSmallLong = 256;
+__device__ inline void sort_members(uint2 *member, uint32_t n) {
+  uint32_t size = 2;
+  while (size < n) size <<= 1;
+  for (uint32_t i = threadIdx.x; i < size; i += kSmallBlock)
+    if (i >= n) member[i] = make_uint2(0xffffffffu, 0xffffffffu);
+  __syncthreads();
+  for (uint32_t run = 2; run <= size; run <<= 1)
+    for (uint32_t step = run >> 1; step; step >>= 1) {
+      for (uint32_t t = threadIdx.x; t < size / 2; t += kSmallBlock) {
+        const uint32_t i = 2 * t - (t & (step - 1)), k = i + step;
+        const uint2 x = member[i], y = member[k];
+        if ((order_key(x) > order_key(y)) == ((i & run) == 0)) {
+          member[i] = y;
+          member[k] = x;
+        }
+      }
+      // steps up to 32 stay within the 64 places of a warp
+      if (step > 32 || (step == 1 && run >= 64)) __syncthreads();
+      else __syncwarp();
+    }
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(kSmallBlock) k_tree_small(FrameTreesView T, TreeSet S,
                                                             const float4 *bb, float pad) {
   extern __shared__ __align__(16) unsigned char s_raw[];
@@ -351,6 +440,7 @@ __global__ void __launch_bounds__(kSmallBlock) k_tree_small(FrameTreesView T, Tr
     }
   }
   __syncthreads();
+  bool sorts;  // some bin is long
   {  // bins' counts to first positions, four bins a thread
     const uint4 c = reinterpret_cast<const uint4 *>(s.first)[tid];
     const uint32_t sum = c.x + c.y + c.z + c.w;
@@ -360,7 +450,7 @@ __global__ void __launch_bounds__(kSmallBlock) k_tree_small(FrameTreesView T, Tr
       if (lane >= (uint32_t)o) incl += y;
     }
     if (lane == 31) s.warp[warp] = incl;
-    __syncthreads();
+    sorts = __syncthreads_or(max(max(c.x, c.y), max(c.z, c.w)) > kSmallLong);
     uint32_t run = incl - sum;
     for (uint32_t w = 0; w < warp; w++) run += s.warp[w];
     reinterpret_cast<uint4 *>(s.first)[tid] =
@@ -373,14 +463,15 @@ __global__ void __launch_bounds__(kSmallBlock) k_tree_small(FrameTreesView T, Tr
     if (e < t.n) s.member[s.first[code[q] >> kTreeBinShift] + slot[q]] = make_uint2(code[q], e);
   }
   __syncthreads();
+  if (sorts) sort_members(s.member, t.n);
   for (uint32_t i = tid; i < t.n; i += kSmallBlock) {
     const uint2 me = s.member[i];
-    const uint32_t bin = me.x >> kTreeBinShift;
-    const uint32_t b0 = s.first[bin], b1 = bin + 1u < kTreeBins ? s.first[bin + 1u] : t.n;
-    uint32_t at = b0;
-    for (uint32_t q = b0; q < b1; q++) {
-      const uint2 m = s.member[q];
-      at += m.x < me.x || (m.x == me.x && m.y < me.y) ? 1u : 0u;  // equal codes by index
+    uint32_t at = i;
+    if (!sorts) {
+      const uint32_t bin = me.x >> kTreeBinShift;
+      const uint32_t b0 = s.first[bin], b1 = bin + 1u < kTreeBins ? s.first[bin + 1u] : t.n;
+      at = b0;
+      for (uint32_t q = b0; q < b1; q++) at += order_key(s.member[q]) < order_key(me) ? 1u : 0u;
     }
     float4 a, b;
     corners(me.y, a, b);

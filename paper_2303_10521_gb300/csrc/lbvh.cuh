@@ -40,13 +40,27 @@ __device__ inline uint32_t frame_code_of(float4 a, float4 b, const float4 *bb) {
   return (uint32_t)morton_code<kMortonBitsDyn>(
       make_float3(0.5f * (a.x + b.x), 0.5f * (a.y + b.y), 0.5f * (a.z + b.z)), bb);
 }
+// at[bin]++ for every calling lane, its place among them returned.  The lanes of
+// the first lane's bin add together: in a crowd they are most of the warp, and
+// atomics on one address complete one after the other (32k of them took 33 us).
+// Finding every lane's peers (match) cost a spread frame 4 us.
+__device__ inline uint32_t add_one(uint32_t *at, uint32_t bin) {
+  const uint32_t lane = threadIdx.x & 31u, all = __activemask();
+  const uint32_t lead = __ffs(all) - 1u;
+  const uint32_t peers = __ballot_sync(all, bin == __shfl_sync(all, bin, lead));
+  const bool together = peers >> lane & 1u;
+  uint32_t place = 0;
+  if (!together || lane == lead) place = atomicAdd(at + bin, together ? (uint32_t)__popc(peers) : 1u);
+  const uint32_t base = __shfl_sync(all, place, lead);
+  return together ? base + __popc(peers & ((1u << lane) - 1u)) : place;
+}
 // The code of primitive i kept and counted in its bin (f.count zero before).
 __device__ inline void frame_code(const FrameTreesBuf &f, uint32_t i, bool vehicle, float4 a,
                                   float4 b, const float4 *bb) {
   const uint32_t code = frame_code_of(a, b, bb);
   f.code[i] = code;
-  f.code[f.cap + i] = atomicAdd(f.count + (code >> kTreeBinShift), 1u);
-  if (vehicle) atomicAdd(f.count + kTreeBins + (code >> kTreeBinShift), 1u);
+  f.code[f.cap + i] = add_one(f.count, code >> kTreeBinShift);
+  if (vehicle) add_one(f.count + kTreeBins, code >> kTreeBinShift);
 }
 
 // Inner node i in [0, n-2] of the radix tree over the sorted keys k: its
