@@ -122,7 +122,7 @@ void launch_evicted(const Counters *c, uint32_t *out, cudaStream_t s) {
   emrt::note_launch(), k_evicted<<<1, 1, 0, s>>>(c, out);
 }
 
-cudaError_t ensure_cand(emrt_scene_s *s, uint64_t need) {
+cudaError_t ensure_cand(emrt_scene_s *s, uint64_t need, cudaStream_t st) {
   if (need <= s->cand_cap && s->cand) return cudaSuccess;
   s->cand_cap = 0;
   uint64_t c = 0;
@@ -132,14 +132,14 @@ cudaError_t ensure_cand(emrt_scene_s *s, uint64_t need) {
   e = grow(&s->cand, c, cap * 8); if (e) return e; c = 0;
   e = grow(&s->uniq, c, cap * 8); if (e) return e; c = 0;
   e = grow(&s->head, c, cap); if (e) return e; c = 0;
-  e = grow(&s->pos, c, cap); if (e) return e; c = 0;
+  e = grow(&s->pos, c, cap + pair_slots(cap)); if (e) return e; c = 0;
+  s->pair_table = s->pos + cap;
+  e = zero_table(s->pair_table, cap, st); if (e) return e;
   e = grow(&s->apts, c, cap * (EMRT_MAX_DEPTH + 2)); if (e) return e; c = 0;
   for (int k = 0; k < 2; k++) {
     e = grow(&s->keys[k], c, cap); if (e) return e; c = 0;
     e = grow(&s->vals[k], c, cap); if (e) return e; c = 0;
   }
-  e = grow(&s->pair_table, c, pair_slots(cap)); if (e) return e;
-  e = zero_table(s->pair_table, cap); if (e) return e;
   s->cand_cap = (uint32_t)cap;
   return cudaSuccess;
 }
@@ -325,7 +325,7 @@ void emrt_scene_destroy(emrt_scene s) {
   for (int k = 0; k < 2; k++) { cudaFree(s->rkeys[k]); cudaFree(s->rvals[k]); }
   cudaFree(s->cand); cudaFree(s->uniq); cudaFree(s->head); cudaFree(s->pos); cudaFree(s->apts);
   for (int k = 0; k < 2; k++) { cudaFree(s->keys[k]); cudaFree(s->vals[k]); }
-  cudaFree(s->pair_count); cudaFree(s->pair_off); cudaFree(s->pair_table);
+  cudaFree(s->pair_count); cudaFree(s->pair_off);
   cudaFree(s->contrib);
   for (int k = 0; k < 4; k++)
     if (s->ev[k]) cudaEventDestroy(s->ev[k]);
@@ -542,7 +542,7 @@ emrt_status run_trace(emrt_scene_s *s, const emrt_trace_params *p, uint64_t coun
   // a rediscovery also concatenates the cache with the new paths in the
   // candidate scratch
   want = merge_cache ? want + out->capacity : std::max<uint64_t>(want, out->capacity);
-  CK(ensure_cand(s, want));
+  CK(ensure_cand(s, want, st));
   const PairSpace pairs = pair_space(s->n_tx, s->n_rx);
   cudaMemsetAsync(s->pair_count, 0, sizeof(uint32_t) * pair_words(pairs.n_pairs), st);
   // counters: keep the error word, clear the rest
@@ -753,7 +753,7 @@ emrt_status emrt_revalidate(emrt_scene s, emrt_paths *cache, uint32_t flags, emr
   if (!s || check_paths(cache) != EMRT_OK) return EMRT_ERR_INVALID_ARG;
   if (!s->updated) return EMRT_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
-  CK(ensure_cand(s, std::max<uint64_t>(s->want_cand, cache->capacity)));
+  CK(ensure_cand(s, std::max<uint64_t>(s->want_cand, cache->capacity), st));
   revalidate_with(s, cache, flags, st, s->uniq, s->partial, s->apts, s->cand_cap, s->ctr);
   CK(cudaGetLastError());
   return EMRT_OK;
@@ -775,7 +775,7 @@ emrt_status emrt_cache_merge(emrt_scene s, emrt_paths *cache, const emrt_paths *
   if (!s->updated) return EMRT_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
   CK(ensure_cand(s, std::max<uint64_t>(s->want_cand,
-                                       (uint64_t)cache->capacity + fresh->capacity)));
+                                       (uint64_t)cache->capacity + fresh->capacity), st));
   Counters *c = s->ctr;
   uint32_t nf = s->Fs + 6 * s->V;
   KeyLayout kl = key_layout(s->n_tx, s->n_rx, nf + 1, EMRT_MAX_DEPTH);
@@ -943,7 +943,7 @@ emrt_status emrt_refresh_schedule(emrt_scene s, float *state, uint8_t *los_ref, 
   if (!s->updated) return EMRT_ERR_STATE;
   cudaStream_t st = (cudaStream_t)stream;
   const uint64_t pairs = (uint64_t)s->n_tx * s->n_rx;
-  CK(ensure_cand(s, std::max<uint64_t>(s->want_cand, pairs)));
+  CK(ensure_cand(s, std::max<uint64_t>(s->want_cand, pairs), st));
   Counters *c = s->ctr;
   GeomView g = geom(s);
   // line of sight of every pair: its direct path through the acceptance

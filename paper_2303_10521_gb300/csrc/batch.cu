@@ -37,7 +37,7 @@ struct emrt_batch_s {
   uint32_t *cand = nullptr, *uniq = nullptr, *pos = nullptr;
   float4 *apts = nullptr;  // acceptance scratch (reflection points)
   uint32_t *pair_count = nullptr, *pair_off = nullptr;  // candidates of every (scene, tx, rx)
-  uint32_t *pair_table = nullptr;
+  uint32_t *pair_table = nullptr;  // long lists' table (behind pos)
   uint32_t n_pairs = 0, pair_shift = 0;  // see PairSpace
   Counters *ctr = nullptr;
   uint32_t *hist = nullptr, *partial = nullptr;
@@ -65,22 +65,21 @@ emrt_status st_of(cudaError_t e) {
 
 void free_scratch(emrt_batch_s *b) {
   cudaFree(b->cand); cudaFree(b->uniq); cudaFree(b->pos); cudaFree(b->apts);
-  cudaFree(b->pair_table);
   b->cand = b->uniq = b->pos = b->pair_table = nullptr;
   b->apts = nullptr;
   b->cand_cap = 0;
 }
 
-cudaError_t alloc_cand(emrt_batch_s *b, uint64_t cap) {
+cudaError_t alloc_cand(emrt_batch_s *b, uint64_t cap, cudaStream_t st) {
   free_scratch(b);
   cap = std::max<uint64_t>(cap, 1024);
   cudaError_t e;
   if ((e = cudaMalloc(&b->cand, 32 * cap))) return e;
   if ((e = cudaMalloc(&b->uniq, 32 * cap))) return e;
-  if ((e = cudaMalloc(&b->pos, 4 * cap))) return e;
+  if ((e = cudaMalloc(&b->pos, sizeof(uint32_t) * (cap + pair_slots(cap))))) return e;
+  b->pair_table = b->pos + cap;
+  if ((e = zero_table(b->pair_table, cap, st))) return e;
   if ((e = cudaMalloc(&b->apts, sizeof(float4) * (EMRT_MAX_DEPTH + 2) * cap))) return e;
-  if ((e = cudaMalloc(&b->pair_table, sizeof(uint32_t) * pair_slots(cap)))) return e;
-  if ((e = zero_table(b->pair_table, cap))) return e;
   b->cand_cap = (uint32_t)cap;
   return cudaSuccess;
 }
@@ -318,7 +317,7 @@ emrt_status emrt_batch_create(const emrt_scene *scenes, uint32_t n, const emrt_t
   uint64_t want = 0;
   for (uint32_t i = 0; i < n; i++)
     want += 4ull * b->scenes[i]->n_tx * b->scenes[i]->n_rx * (b->params[i].max_depth + 1);
-  BCK(alloc_cand(b, std::max<uint64_t>(want, 1u << 16)));
+  BCK(alloc_cand(b, std::max<uint64_t>(want, 1u << 16), st));
   // autotune (or read the cached choice)
   int dev = 0;
   cudaGetDevice(&dev);
@@ -361,7 +360,7 @@ emrt_status emrt_batch_create(const emrt_scene *scenes, uint32_t n, const emrt_t
         Counters h;
         cudaMemcpy(&h, b->ctr, sizeof(Counters), cudaMemcpyDeviceToHost);
         if (h.n_cand > b->cand_cap) {  // grow and retry this variant
-          BCK(alloc_cand(b, (uint64_t)h.n_cand + h.n_cand / 4 + 1024));
+          BCK(alloc_cand(b, (uint64_t)h.n_cand + h.n_cand / 4 + 1024, st));
           v--;
           cudaMemset(b->ctr, 0, sizeof(uint32_t));
           continue;
@@ -498,7 +497,7 @@ emrt_status emrt_batch_trace(emrt_batch b, emrt_stream stream) {
   }
   if (b->want_cand > b->cand_cap) {  // a previous call overflowed: grow, re-capture
     drop_graph(b);
-    BCK(alloc_cand(b, b->want_cand));
+    BCK(alloc_cand(b, b->want_cand, st));
   }
   BCK(cudaStreamSynchronize(st));  // the pinned table may still be read by a copy
   fill_table(b);

@@ -59,7 +59,7 @@ struct emrt_scene_s {
   uint32_t *vals[2] = {nullptr, nullptr};
   // candidates of every (tx, rx) pair: counts and places, for any frame
   uint32_t *pair_count = nullptr, *pair_off = nullptr;
-  uint32_t *pair_table = nullptr;  // long lists' table (pair_slots(cand_cap))
+  uint32_t *pair_table = nullptr;  // long lists' table (behind pos)
   // adjoint scratch
   double *contrib = nullptr;
   uint64_t contrib_cap = 0;

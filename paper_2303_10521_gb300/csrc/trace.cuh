@@ -194,10 +194,9 @@ struct PairBufs {
 // The table has pair_slots(cap) words, zero before and after every dedup.
 constexpr uint32_t kPairLong = 256;
 inline uint64_t pair_slots(uint64_t cap) { return 2 * cap; }
-// a new table's zeros (when it returns they are there for every stream)
-inline cudaError_t zero_table(uint32_t *table, uint64_t cap) {
-  const cudaError_t e = cudaMemset(table, 0, sizeof(uint32_t) * pair_slots(cap));
-  return e ? e : cudaStreamSynchronize(nullptr);
+// the zeros of a new table
+inline cudaError_t zero_table(uint32_t *table, uint64_t cap, cudaStream_t s) {
+  return cudaMemsetAsync(table, 0, sizeof(uint32_t) * pair_slots(cap), s);
 }
 // words at count for n_pairs pairs (count, more, group), and their places
 uint64_t pair_words(uint64_t n_pairs);
