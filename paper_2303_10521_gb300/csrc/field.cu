@@ -6,6 +6,8 @@
 // recomputes a path's points, basis vectors and coefficients instead of
 // storing them and runs the same steps backwards.  Path length and phase are
 // accumulated in FP64 (L / lambda formed in double).
+#include <algorithm>
+
 #include "field.cuh"
 
 namespace emrt {
@@ -718,6 +720,11 @@ __global__ void __launch_bounds__(kGradBlock) k_grad_reduce(GeomView g, MatView 
 // series (two square roots a term) -> 1.42 ms (the FP64 FMAs alone: 0.97 ms).
 // RESIDENT: the whole series of the block fits (n_buf = F); otherwise chunks
 // of n_buf frames and, for the lagged factor, n_buf + kCorrLags frames.
+// Few pairs and many lags: passes of kCorrLags lags go to the grid's second
+// dimension, up to two blocks an SM (each takes its pairs' mean and variance
+// itself, which four blocks an SM do not gain back); a block that takes all
+// passes of one pair leaves 151 SMs idle.  1 pair x 20000 frames x 2001 lags 135 ->
+// 5.9 ms, 64 x 1500 x 1001 2.56 -> 0.40, 500 x 300 x 251 0.173 -> 0.102.
 constexpr int kCorrPairs = 8, kCorrBlock = 128;
 constexpr int kCorrTile = 4;                                    // lag groups per warp
 constexpr int kCorrLags = (kCorrBlock / 32) * kCorrTile * 4;    // lags of one pass
@@ -745,11 +752,13 @@ __global__ void __launch_bounds__(kCorrBlock) k_correlation(const double *h, uin
   const uint32_t pl = lane % kCorrPairs, tq = lane / kCorrPairs;
   const uint32_t p0 = blockIdx.x * kCorrPairs;
   double *s_lag = RESIDENT ? s_g : s_g + n_buf * kCorrPairs;
-  for (uint64_t tb = 0; tb <= L; tb += kCorrLags) {
-    double c[kCorrTile] = {}, s1 = 0.0;
+  const uint64_t first = (uint64_t)blockIdx.y * kCorrLags;
+  for (uint64_t tb = first; tb <= L; tb += (uint64_t)gridDim.y * kCorrLags) {
+    double c[kCorrTile] = {}, s1 = 0.0, s2 = 0.0;
     const uint64_t w0 = tb + warp * (4 * kCorrTile);  // first lag of this warp
-    for (uint32_t t0 = 0; t0 < F; t0 += n_buf) {
-      if (!RESIDENT || tb == 0) {
+    for (uint64_t start = 0; start < F; start += n_buf) {
+      const uint32_t t0 = (uint32_t)start;
+      if (!RESIDENT || tb == first) {
         __syncthreads();
         corr_stage(h, F, P, p0, t0, min(n_buf, F - t0), s_g);
         if (!RESIDENT && t0 + tb < F)
@@ -760,8 +769,11 @@ __global__ void __launch_bounds__(kCorrBlock) k_correlation(const double *h, uin
       const double *ga = s_g + pl;
       // lag j of this lane: w0 + 4 j + tq, its factor gb[(t + 4 j) * kCorrPairs]
       const double *gb = s_lag + (RESIDENT ? w0 : w0 - tb) * kCorrPairs + tq * kCorrPairs + pl;
-      if (tb == 0 && warp == 0)
+      if (tb == first && warp == 0) {
         for (uint32_t t = 0; t < m; t++) s1 += ga[t * kCorrPairs];
+        if (first)  // the block has no lag 0
+          for (uint32_t t = 0; t < m; t++) s2 += ga[t * kCorrPairs] * ga[t * kCorrPairs];
+      }
       // terms of this chunk for each lag: t0 + t + tau < F
       uint32_t n[kCorrTile];
       int groups = 0;  // lag groups of this warp with terms (warp-uniform)
@@ -785,11 +797,11 @@ __global__ void __launch_bounds__(kCorrBlock) k_correlation(const double *h, uin
           for (uint32_t t = done; t < n[j]; t++)
             c[j] += ga[t * kCorrPairs] * gb[(t + 4 * j) * kCorrPairs];
     }
-    if (tb == 0) {
+    if (tb == first) {
       if (warp == 0 && tq == 0) {  // lag 0: the sum of squares
         const double mu = s1 / F;
         s_mu[pl] = mu;
-        s_var[pl] = c[0] / F - mu * mu;
+        s_var[pl] = (first ? s2 : c[0]) / F - mu * mu;
       }
       __syncthreads();
     }
@@ -900,7 +912,9 @@ cudaError_t launch_correlation(const double *h, uint32_t n_frames, uint32_t n_pa
   const cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
   if (e) return e;
-  emrt::note_launch(), kern<<<ceil_div(n_pairs, kCorrPairs), kCorrBlock, smem, s>>>(
+  const uint32_t blocks = ceil_div(n_pairs, kCorrPairs), passes = max_lag / kCorrLags + 1;
+  const uint32_t split = std::max<uint32_t>(1u, std::min<uint32_t>(passes, 2 * 152 / blocks));
+  emrt::note_launch(), kern<<<dim3(blocks, split), kCorrBlock, smem, s>>>(
       h, n_frames, n_pairs, max_lag, n_buf, R);
   return cudaGetLastError();
 }
