@@ -610,12 +610,12 @@ int walk_grid() {
 // n_rx kappa is the expected number of receivers whose sphere a ray across the
 // scene meets.  Walk with the query against without (cities of 10 and 30 blocks,
 // 2e2-1e4 receivers, 1M-32M rays; the two cities' factors, K = 2 / K = 4):
-//   rays  n_rx kappa 1       2.5                     5                       10
-//   1M   1.10-1.18 / 1.03  1.03-1.10 / 0.98-1.01   0.95-0.99 / 0.92-0.93   0.85-0.90 / 0.85-0.87
-//   4M   1.21-1.22 / 1.05  1.12-1.15 / 1.00-1.04   1.06-1.10 / 0.96-1.01   1.01-1.02 / 0.95-0.97
-//   8M   1.21-1.23 / 1.07  1.16-1.18 / 1.04-1.06   1.11-1.14 / 1.02-1.03   1.05-1.07 / 0.98-1.00
-//   16M  1.22-1.24 / 1.08  1.19-1.20 / 1.06-1.08   1.15-1.16 / 1.04-1.05   1.11-1.12 / 1.01-1.02
-//   32M  1.21-1.24 / 1.08  1.19-1.21 / 1.07        1.17-1.19 / 1.05-1.06   1.14-1.15 / 1.03-1.04
+//   rays  n_rx kappa 1            2.5                     5                       10
+//   1M   1.10-1.18 / 1.03       1.03-1.10 / 0.98-1.01   0.95-0.99 / 0.92-0.93   0.85-0.90 / 0.85-0.87
+//   4M   1.21-1.22 / 1.05-1.07  1.12-1.15 / 1.00-1.04   1.06-1.10 / 0.96-1.01   1.01-1.02 / 0.95-0.97
+//   8M   1.21-1.23 / 1.07-1.10  1.16-1.18 / 1.04-1.06   1.11-1.14 / 1.02-1.03   1.05-1.07 / 0.98-1.00
+//   16M  1.22-1.24 / 1.08-1.10  1.19-1.20 / 1.06-1.08   1.15-1.16 / 1.04-1.05   1.11-1.12 / 1.01-1.02
+//   32M  1.21-1.24 / 1.08-1.10  1.19-1.21 / 1.07        1.17-1.19 / 1.05-1.06   1.14-1.15 / 1.03-1.04
 // (fewer rays are bound by their longest chains, which the query makes longer;
 // at 32M rays n_rx kappa of 19 0.94-1.00, of 39 0.77-0.87).
 bool walk_ends_last(uint64_t n_rays_launched, uint32_t n_rx, float kappa) {
