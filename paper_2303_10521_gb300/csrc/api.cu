@@ -123,25 +123,33 @@ void launch_evicted(const Counters *c, uint32_t *out, cudaStream_t s) {
 }
 
 cudaError_t ensure_cand(emrt_scene_s *s, uint64_t need, cudaStream_t st) {
-  if (need <= s->cand_cap && s->cand) return cudaSuccess;
-  s->cand_cap = 0;
-  uint64_t c = 0;
-  cudaError_t e;
-  uint64_t cap = std::max<uint64_t>(need, 1024);
-  if (cap > 0xffffffffull / 2) cap = 0xffffffffull / 2;
-  e = grow(&s->cand, c, cap * 8); if (e) return e; c = 0;
-  e = grow(&s->uniq, c, cap * 8); if (e) return e; c = 0;
-  e = grow(&s->head, c, cap); if (e) return e; c = 0;
-  e = grow(&s->pos, c, cap + pair_slots(cap)); if (e) return e; c = 0;
-  s->pair_table = s->pos + cap;
-  e = zero_table(s->pair_table, cap, st); if (e) return e;
-  e = grow(&s->apts, c, cap * (EMRT_MAX_DEPTH + 2)); if (e) return e; c = 0;
-  for (int k = 0; k < 2; k++) {
-    e = grow(&s->keys[k], c, cap); if (e) return e; c = 0;
-    e = grow(&s->vals[k], c, cap); if (e) return e; c = 0;
+  if (need > s->cand_cap || !s->cand) {
+    s->cand_cap = 0;
+    uint64_t c = 0;
+    cudaError_t e;
+    uint64_t cap = std::max<uint64_t>(need, 1024);
+    if (cap > 0xffffffffull / 2) cap = 0xffffffffull / 2;
+    e = grow(&s->cand, c, cap * 8); if (e) return e; c = 0;
+    e = grow(&s->uniq, c, cap * 8); if (e) return e; c = 0;
+    e = grow(&s->head, c, cap); if (e) return e; c = 0;
+    e = grow(&s->pos, c, cap + pair_slots(cap)); if (e) return e; c = 0;
+    s->pair_table = s->pos + cap;
+    s->pair_table_zero = false;
+    e = grow(&s->apts, c, cap * (EMRT_MAX_DEPTH + 2)); if (e) return e; c = 0;
+    for (int k = 0; k < 2; k++) {
+      e = grow(&s->keys[k], c, cap); if (e) return e; c = 0;
+      e = grow(&s->vals[k], c, cap); if (e) return e; c = 0;
+    }
+    s->cand_cap = (uint32_t)cap;
   }
-  s->cand_cap = (uint32_t)cap;
-  return cudaSuccess;
+  if (s->pair_table_zero) return cudaSuccess;
+  // a new table's zeros: a memset that is only recorded into a caller's graph
+  // leaves the table as it is, so every call issues one until one runs
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(st, &capture);
+  if (!e) e = zero_table(s->pair_table, s->cand_cap, st);
+  s->pair_table_zero = !e && capture == cudaStreamCaptureStatusNone;
+  return e;
 }
 
 // The pairs of n_tx transmitters and n_rx receivers.

@@ -60,6 +60,7 @@ struct emrt_scene_s {
   // candidates of every (tx, rx) pair: counts and places, for any frame
   uint32_t *pair_count = nullptr, *pair_off = nullptr;
   uint32_t *pair_table = nullptr;  // long lists' table (behind pos)
+  bool pair_table_zero = false;    // its zeros have been issued
   // adjoint scratch
   double *contrib = nullptr;
   uint64_t contrib_cap = 0;
